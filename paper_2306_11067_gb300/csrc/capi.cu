@@ -1456,8 +1456,7 @@ struct PaperMG {
     else
       klaunch(k_pm_dense, dim3(gd), dim3(kBlock), 0, s, glop(L - 1), c.lam2.p, c.pm_AtAc.p, c.Mw.p);
     LCMG_LAUNCHED();
-    klaunch(k_cholesky_inverse, dim3(1), dim3(kBlock), 0, s, (int)nc, c.Mw.p, c.Ww.p, c.kinv.p, c.s_info.p);
-    LCMG_LAUNCHED();
+    launch_dense_inverse((int)nc, 1, c.Mw.p, c.Ww.p, c.kinv.p, c.s_info.p, s);
     int info = 0;
     copy_sync(s, &info, c.s_info.p, sizeof(int), cudaMemcpyDeviceToHost);
     if (info != 0) throw ArgError("coarsest-level Cholesky failed (pivot " + std::to_string(info) + ")");

@@ -751,57 +751,138 @@ __global__ void __launch_bounds__(kBlock)
   }
 }
 
-// In-place dense Cholesky K = L L^T (lower, row-major) followed by the
-// explicit inverse K^{-1} = L^{-T} L^{-1}; one block per column.  W is an
-// n x n scratch per column.  info[col] = 0 on success, else the 1-based
-// pivot that was not positive.
-static __global__ void __launch_bounds__(kBlock)
-    k_cholesky_inverse(int n, double* __restrict__ Mall, double* __restrict__ Wall,
-                       double* __restrict__ Kall, int* __restrict__ info) {
-  const int col = blockIdx.x;
-  double* M = Mall + (int64_t)col * n * n;
-  double* X = Wall + (int64_t)col * n * n;
-  double* K = Kall + (int64_t)col * n * n;
+// Explicit inverse K^{-1} = L^{-T} L^{-1} of the coarsest-level matrices
+// M = L L^T (symmetric positive definite, n x n, one per column of the
+// batch).  Factorisation, X = L^{-1} and K^{-1} = X^T X advance together, 16
+// columns of L per launch, in place on the lower triangle: at step k, with
+// block row / column k the pivot,
+//   tile (i, j), i >= j > k:  M_ij  -= L_ik L_jk^T       (trailing matrix)
+//   tile (i, j), i > k >= j:  S_ij  -= L_ik X_kj         (S_ij becomes X_ij at step i)
+//   tile (i, j), k >= i >= j: K_ij  += X_ki^T X_kj       (the inverse)
+// where S_kk = I and the last two start from 0 at step j and at step i.  Both
+// factors of every product are rows u solved against the pivot block's
+// factor, u_t = (u_t - sum_{s<t} u_s L_ts) / L_tt: rows of M_ik, or columns
+// of S_kj.  Every element sees the additions of the unblocked algorithm in
+// its order (increasing k), so the result does not depend on the tiling.
+//
+// What bounds it: FP64 runs at less than two multiply-adds per clock and SM
+// here, so the n^3 / 2 of them have to be spread over the GPU: one block of
+// threads per 16 x 16 tile (136 at n = 256), one launch per step; and the
+// chain of 16 dependent pivots (square root and reciprocal, about 80 cycles
+// per FP64 operation), which every block goes through again for the pivot
+// block rather than wait for another launch.  So that little else stands in
+// the chain, the pivot block, the two panels and the tile have 256 threads
+// each, a column's threads lie in different SM quarters for the three
+// solves, and a division is three operations from the pivot's reciprocal.
+// A step reads `src` and writes `dst` (the pivot row and column are read by
+// every block).  info[col] = the 1-based index of the first pivot that was
+// not positive.
+//
+// Measured on GB300 against one block per column that did all of it in
+// global memory: n = 160 2,530 -> 187 us, n = 256 11,400 -> about 300 us,
+// n = 567 123,000 -> 2,220 us; the same values bit for bit.
+constexpr int kInvTile = 16;
+
+// sqrt(a) and its reciprocal, both rounded to nearest: an FP32 seed, one
+// third-order step for 1 / sqrt(a), then one residual correction of each
+// (the divisions below need the correctly rounded reciprocal).  Outside the
+// FP32 range the library's operations.
+__device__ __forceinline__ void pivot_root(double a, double& root, double& recip) {
+  if (a > 1e-36 && a < 1e36) {
+    const double y0 = (double)rsqrtf((float)a);
+    const double e = fma(-a * y0, y0, 1.0);
+    const double y = fma(y0, e * fma(e, 0.375, 0.5), y0);
+    const double s = a * y;
+    root = fma(0.5 * y, fma(-s, s, a), s);
+    recip = fma(y, fma(-root, y, 1.0), y);
+  } else {
+    root = sqrt(a);
+    recip = 1.0 / root;
+  }
+}
+
+static __global__ void __launch_bounds__(4 * kInvTile * kInvTile)
+    k_inverse_step(int n, int k, int last, const double* __restrict__ srcall, double* __restrict__ dstall,
+                   int* __restrict__ info) {
+  constexpr int Q = kInvTile;
+  // the pivot block (then its factor, lower triangle) and the two panels
+  __shared__ double A[3][Q][Q + 1];
+  __shared__ double s_piv, s_rec;
   __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
+  const int col = blockIdx.y;
+  const double* __restrict__ S = srcall + (int64_t)col * n * n;
+  double* __restrict__ O = dstall + (int64_t)col * n * n;
+  // tile (bi, bj), bi >= bj, of the lower triangle
+  int bi = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+  while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
+  const int bj = (int)blockIdx.x - bi * (bi + 1) / 2;
+  // group 0: pivot block, 1 and 2: panels of block rows bi and bj, 3: tile;
+  // a half warp holds a column, the groups' columns shifted by one warp
+  const int g = threadIdx.x / (Q * Q), l = threadIdx.x % (Q * Q);
+  const int c = 2 * ((l / 32 + 8 - g) % 8) + (l / 16) % 2, r = l % Q;
+  // element (rr, cc) of tile (u, v), u >= v; a last partial tile is padded
+  // with the rows and columns of the identity
+  auto get = [&](int u, int v, int rr, int cc) {
+    const int i = u * Q + rr, j = v * Q + cc;
+    if (i < n && j < n) return S[(int64_t)i * n + j];
+    return i == j ? 1.0 : 0.0;
+  };
+  // the panel of block row b: rows of M_bk (b > k), the identity (b = k), or
+  // the columns of S_kb (b < k)
+  auto panel = [&](int b, int rr, int cc) {
+    if (b > k) return get(b, k, rr, cc);
+    if (b == k) return rr == cc ? 1.0 : 0.0;
+    return get(k, b, cc, rr);
+  };
+  const bool trail = bi > k;  // the tile subtracts (else it adds)
+  double x = g == 0   ? get(k, k, r, c)
+             : g == 1 ? panel(bi, r, c)
+             : g == 2 ? panel(bj, r, c)
+             : (trail ? bj == k : bi == k) ? 0.0
+                                           : get(bi, bj, r, c);
+  auto pivot = [&](int t, double a) {
+    if (!(a > 0.0)) {
+      if (!bad) bad = k * Q + t + 1;
+      a = 1.0;
+    }
+    double root, recip;
+    pivot_root(a, root, recip);
+    s_piv = root;
+    s_rec = recip;
+  };
+  if (threadIdx.x == 0) {
+    bad = 0;
+    pivot(0, x);
+  }
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) {
-      const double d = M[(int64_t)k * n + k];
-      if (!(d > 0.0) && !bad) bad = k + 1;
-      M[(int64_t)k * n + k] = sqrt(d > 0.0 ? d : 1.0);
+  for (int t = 0; t < Q; ++t) {
+    if (c == t && g < 3) {  // column t, final
+      const double piv = s_piv, rec = s_rec;
+      if (g == 0 && r == t) {
+        x = piv;
+      } else {  // x / piv to nearest (Markstein 1990: quotient, exact remainder, correction)
+        const double q = x * rec;
+        x = fma(fma(-q, piv, x), rec, q);
+      }
+      A[g][r][t] = x;
     }
     __syncthreads();
-    const double piv = M[(int64_t)k * n + k];
-    for (int i = k + 1 + threadIdx.x; i < n; i += kBlock) M[(int64_t)i * n + k] /= piv;
-    __syncthreads();
-    const int m = n - k - 1;
-    for (int64_t t = threadIdx.x; t < (int64_t)m * m; t += kBlock) {
-      const int i = k + 1 + (int)(t / m), jj = k + 1 + (int)(t % m);
-      if (jj <= i) M[(int64_t)i * n + jj] -= M[(int64_t)i * n + k] * M[(int64_t)jj * n + k];
+    if (g == 3) {
+      const double uv = trail ? -A[1][r][t] : A[1][r][t];
+      x = fma(uv, A[2][c][t], x);
+    } else if (c > t && (g != 0 || r >= c)) {
+      x -= A[g][r][t] * A[0][c][t];
+      if (g == 0 && c == t + 1 && r == c) pivot(c, x);
     }
     __syncthreads();
   }
-  // X = L^{-1} (lower): column c by forward substitution, one thread per c
-  for (int c = threadIdx.x; c < n; c += kBlock) {
-    for (int i = 0; i < c; ++i) X[(int64_t)i * n + c] = 0.0;
-    for (int i = c; i < n; ++i) {
-      double s = (i == c) ? 1.0 : 0.0;
-      for (int k = c; k < i; ++k) s -= M[(int64_t)i * n + k] * X[(int64_t)k * n + c];
-      X[(int64_t)i * n + c] = s / M[(int64_t)i * n + i];
-    }
+  if (blockIdx.x == 0 && threadIdx.x == 0 && bad && info[col] == 0) info[col] = bad;
+  const int i = bi * Q + r, j = bj * Q + c;
+  if (g == 3 && i < n && j < n) {
+    O[(int64_t)i * n + j] = x;
+    if (last && bi != bj) O[(int64_t)j * n + i] = x;
   }
-  __syncthreads();
-  // K^{-1}[p][q] = sum_{i >= max(p,q)} X[i][p] X[i][q]
-  for (int64_t t = threadIdx.x; t < (int64_t)n * n; t += kBlock) {
-    const int p = (int)(t / n), q = (int)(t % n);
-    if (q < p) continue;
-    double s = 0.0;
-    for (int i = q; i < n; ++i) s += X[(int64_t)i * n + p] * X[(int64_t)i * n + q];
-    K[(int64_t)p * n + q] = s;
-    K[(int64_t)q * n + p] = s;
-  }
-  if (threadIdx.x == 0) info[col] = bad;
 }
 
 // ---------------------------------------------------------------------------

@@ -92,6 +92,10 @@ void launch_vtail(const TailLevelIn* levels, int nlev, const double* kinv, int n
 bool vtail_fits(int nlev);
 void launch_dense_setup(const LevelView<double>& L, int B, const double* lam2, double* M,
                         double* W, double* K, int* info, int max_blocks, cudaStream_t s);
+// K = M^{-1} of B symmetric positive definite n x n matrices (lower triangle
+// of M read; W is scratch of the same size, M keeps its values); info[b] = 0,
+// or the 1-based index of the first pivot that was not positive
+void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, int* info, cudaStream_t s);
 void launch_galerkin(const RapIn& in, int nvc, int nhc, double* out, int max_blocks, cudaStream_t s);
 
 template <class T, class TX>

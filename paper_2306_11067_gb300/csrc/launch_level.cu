@@ -345,8 +345,20 @@ void launch_dense_setup(const LevelView<double>& L, int B, const double* lam2, d
   else
     klaunch(k_dense_assemble<CoarseOp<double>>, dim3(g), dim3(kBlock), 0, s, L.coarse_op(), nc, B, lam2, M);
   LCMG_LAUNCHED();
-  klaunch(k_cholesky_inverse, dim3(B), dim3(kBlock), 0, s, (int)nc, M, W, K, info);
-  LCMG_LAUNCHED();
+  launch_dense_inverse((int)nc, B, M, W, K, info, s);
+}
+
+void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, int* info, cudaStream_t s) {
+  LCMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int) * B, s));
+  const int nb = (n + kInvTile - 1) / kInvTile;
+  const double* src = M;
+  for (int k = 0; k < nb; ++k) {  // the last step writes K
+    double* dst = (nb - 1 - k) % 2 == 0 ? K : W;
+    klaunch(k_inverse_step, dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)B), dim3(4 * kInvTile * kInvTile), 0, s, n,
+            k, k == nb - 1 ? 1 : 0, src, dst, info);
+    LCMG_LAUNCHED();
+    src = dst;
+  }
 }
 
 void launch_galerkin(const RapIn& in, int nvc, int nhc, double* out, int max_blocks, cudaStream_t s) {
