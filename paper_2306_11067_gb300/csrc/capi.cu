@@ -2271,13 +2271,15 @@ static void set_separable(lcmg_ctx* c, const std::vector<double>& fv, const std:
   c->sp_ha = sep_pass_corr(fh, false);
   c->sp_vat = sep_pass_corr(fv, true);
   c->sp_hat = sep_pass_corr(fh, true);
-  auto up = [&](const std::vector<double>& d, DevBuf<double>& b64, DevBuf<float>& b32) {
+  auto up = [&](const SepPass& p, DevBuf<double>& b64, DevBuf<float>& b32) {
+    std::vector<double> d(p.d);
+    d.insert(d.end(), p.e.begin(), p.e.end());
     std::vector<float> f32(d.begin(), d.end());
     copy_sync(c->stream, b64.need(d.size()), d.data(), sizeof(double) * d.size(), cudaMemcpyHostToDevice);
     copy_sync(c->stream, b32.need(d.size()), f32.data(), sizeof(float) * d.size(), cudaMemcpyHostToDevice);
   };
-  up(c->sp_vt.d, c->sep_dv64, c->sep_dv32);
-  up(c->sp_ht.d, c->sep_dh64, c->sep_dh32);
+  up(c->sp_vt, c->sep_dv64, c->sep_dv32);
+  up(c->sp_ht, c->sep_dh64, c->sep_dh32);
   const std::vector<double> dv = sep_diag(c->sp_vt, c->nv), dh = sep_diag(c->sp_ht, c->nh);
   DevBuf<double> ddv, ddh;
   copy_sync(c->stream, ddv.need(dv.size()), dv.data(), sizeof(double) * dv.size(), cudaMemcpyHostToDevice);

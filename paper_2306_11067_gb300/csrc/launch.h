@@ -126,6 +126,7 @@ struct SepPass {
   std::vector<double> c;
   int nlo = 0, nhi = 0;
   std::vector<double> d;
+  std::vector<double> e;  // the whole rows of those outputs (c + d) and the interior row, or empty
 };
 // the 1-D correlation with taps f (2r + 1 values) or its transpose
 SepPass sep_pass_corr(const std::vector<double>& f, bool transpose);
@@ -133,7 +134,7 @@ SepPass sep_pass_corr(const std::vector<double>& f, bool transpose);
 SepPass sep_pass_ata(const std::vector<double>& f, int len);
 // the diagonal of a sep_pass_ata pass (len values)
 std::vector<double> sep_diag(const SepPass& p, int len);
-// device form of a pass whose correction rows live at d_dev
+// device form of a pass whose tables d, then e, live at d_dev
 template <class T>
 Band<T> make_band(const SepPass& p, const T* d_dev);
 // one pass over every line of an n_v x n_h image and B interleaved columns

@@ -46,7 +46,8 @@ SepPass sep_pass_ata(const std::vector<double>& f, int len) {
   }
   p.nlo = std::min(r, len);
   p.nhi = std::min(r, len - p.nlo);
-  auto exact_row = [&](int i, std::vector<double>& row) {
+  p.e.assign((size_t)(p.nlo + p.nhi + 1) * taps, 0.0);
+  auto exact_row = [&](int i, std::vector<double>& row, double* whole) {
     for (int k = -H; k <= H; ++k) {
       double s = 0.0;
       if (i + k >= 0 && i + k < len)
@@ -55,18 +56,20 @@ SepPass sep_pass_ata(const std::vector<double>& f, int len) {
       // the interior coefficient applies to in(i + k) only where it exists
       const double interior = (i + k >= 0 && i + k < len) ? p.c[k + H] : 0.0;
       row[k + H] = s - interior;
+      whole[k + H] = s;
     }
   };
   p.d.assign((size_t)(p.nlo + p.nhi) * taps, 0.0);
   std::vector<double> row(taps);
   for (int i = 0; i < p.nlo; ++i) {
-    exact_row(i, row);
+    exact_row(i, row, p.e.data() + (size_t)i * taps);
     std::copy(row.begin(), row.end(), p.d.begin() + (size_t)i * taps);
   }
   for (int q = 0; q < p.nhi; ++q) {
-    exact_row(len - p.nhi + q, row);
+    exact_row(len - p.nhi + q, row, p.e.data() + (size_t)(p.nlo + q) * taps);
     std::copy(row.begin(), row.end(), p.d.begin() + (size_t)(p.nlo + q) * taps);
   }
+  std::copy(p.c.begin(), p.c.end(), p.e.end() - taps);
   return p;
 }
 
@@ -89,10 +92,14 @@ Band<T> make_band(const SepPass& p, const T* d_dev) {
   b.nlo = p.d.empty() ? 0 : p.nlo;
   b.nhi = p.d.empty() ? 0 : p.nhi;
   b.d = p.d.empty() ? nullptr : d_dev;
+  b.e = p.d.empty() ? nullptr : d_dev + p.d.size();
   return b;
 }
 
-// blocks of k_band resident at once on the current device
+// largest FP32 pass (points x columns) that runs with one output per thread
+constexpr int64_t kBandDirectMax = 256 * 256;
+
+// blocks of a banded pass resident at once on the current device
 template <class K>
 static int band_resident(K kern, size_t smem) {
   static std::mutex mu;
@@ -126,43 +133,55 @@ static int band_go(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* ou
   return (int)blocks;
 }
 
-// the A^T A passes of radii 4, 9 and 15 (17, 37 and 61 taps) with their tap
-// count compiled in; every other pass with the chunked loop
+template <class T, class TO, int DIR, int EPI>
+static int band_direct_go(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop,
+                          const T* P, const T* C, const double* lam2, const double* bvec, double* part,
+                          int max_blocks, cudaStream_t s) {
+  auto k = k_band_direct<T, TO, DIR, EPI>;
+  const int64_t n = (int64_t)nv * nh;
+  // small images in blocks of two warps, so that they spread over more SMs
+  const int threads = n <= 64 * 1024 ? 64 : kBandThreads;
+  int64_t blocks = std::min<int64_t>((n + threads - 1) / threads, band_resident(k, 0));
+  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, max_blocks));
+  klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(threads), 0, s, nv, nh, B, bd, in, out, fop, P, C, lam2, bvec,
+          part);
+  LCMG_LAUNCHED();
+  return (int)blocks;
+}
+
+// FP64, and FP32 images whose tiles would leave most of the GPU idle: one
+// output per thread.  FP32 otherwise: staged tiles, with the tap count of
+// the A^T A passes of radii 4, 9 and 15 (17, 37 and 61 taps) compiled in,
+// every other pass with the chunked loop.
 template <class T, class TO, int DIR, int EPI>
 int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
                 const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s) {
-  constexpr bool kHot = EPI != BAND_RESID2 && !(std::is_same<T, double>::value && DIR == 1 && EPI == BAND_STORE);
-  if constexpr (kHot) {
+  if constexpr (std::is_same<T, double>::value) {
+    return band_direct_go<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+  } else {
+    if ((int64_t)nv * nh * B <= kBandDirectMax)
+      return band_direct_go<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
     switch (2 * bd.H + 1) {
       case 17: return band_go<T, TO, DIR, EPI, 17>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
       case 37: return band_go<T, TO, DIR, EPI, 37>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
       case 61: return band_go<T, TO, DIR, EPI, 61>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-      default: break;
+      default: return band_go<T, TO, DIR, EPI, 0>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
     }
   }
-  return band_go<T, TO, DIR, EPI, 0>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
 }
 
 template <class T, class TO, int DIR, int EPI>
 static void band_optin() {
   const int bytes = (int)band_smem_bytes<T>((2 * kBandMaxH + 1 + kBandChunk - 1) / kBandChunk);
   LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  constexpr bool kHot = EPI != BAND_RESID2 && !(std::is_same<T, double>::value && DIR == 1 && EPI == BAND_STORE);
-  if constexpr (kHot) {
-    LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 17>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 37>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 61>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  }
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 17>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 37>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 61>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
 }
 
 void prepare_band() {
   band_optin<float, float, 0, BAND_STORE>();
   band_optin<float, float, 1, BAND_NORMAL>();
-  band_optin<double, double, 0, BAND_STORE>();
-  band_optin<double, double, 1, BAND_STORE>();
-  band_optin<double, double, 1, BAND_NORMAL>();
-  band_optin<double, double, 1, BAND_RESID2>();
-  band_optin<double, double, 1, BAND_TRUERES>();
 }
 
 void launch_sep_diag(int nv, int nh, const double* dv, const double* dh, double* diag, int max_blocks,

@@ -53,6 +53,8 @@ struct Band {
   int nch;             // chunks of kBandChunk taps: ceil((2H + 1) / 8)
   int nlo, nhi;
   const T* d;          // (nlo + nhi) x (2H + 1) corrections, or null
+  const T* e;          // the whole coefficient rows c + d of those outputs and, last, the
+                       // interior row c: (nlo + nhi + 1) x (2H + 1), or null
   T c[kBandMaxTaps];   // zero beyond 2H
 };
 
@@ -236,6 +238,104 @@ __global__ void __launch_bounds__(kBandThreads)
     if (threadIdx.x == 0) {
       double s = 0.0;
       for (int k = 0; k < kBandThreads / 32; ++k) s += sred[k];
+      part[(int64_t)blockIdx.x * B + col] = s;
+    }
+  }
+}
+
+// The same pass with one output per thread and no staging: a thread reads
+// its 2H + 1 samples through L1 (consecutive lanes consecutive points along
+// the contiguous axis, so every tap of a warp is one or two lines).  Rows
+// near the ends of the line take their whole coefficient row from bd.e, in
+// one sum; a warp that holds both kinds of rows reads the table for all of
+// its lanes (the last row of the table is the interior one).
+//
+// In FP64 the multiply-adds bound it, not the loads: the pipe takes 19
+// cycles per warp instruction, in which L1 serves several taps, so the
+// staged tiles of k_band only cost barriers there; and on small images
+// k_band has too few tiles to fill the GPU (2 blocks at 64 x 64) where one
+// output per thread uses it all.  Measured on GB300, both passes of A^T A in
+// FP64, k_band -> this: 64 x 64, 37 taps 55 + 64 -> 4.5 + 9.6 us; 240 x 176,
+// 29 and 25 taps 44 + 56 -> 4.5 + 9.3 us; 1024 x 1024, 61 taps 164 + 190 ->
+// 128 + 161 us (the multiply-adds alone take 120 each).
+template <class T, class TO, int DIR, int EPI>
+__global__ void __launch_bounds__(kBandThreads)
+    k_band_direct(int nv, int nh, int B, const __grid_constant__ Band<T> bd, const T* __restrict__ in,
+                  TO* __restrict__ out, FineOp<T> fop, const T* __restrict__ P, const T* __restrict__ C,
+                  const double* __restrict__ lam2, const double* __restrict__ bvec, double* __restrict__ part) {
+  __shared__ double sred[kBandThreads / 32];
+  const int col = blockIdx.y;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int H = bd.H, taps = 2 * H + 1;
+  const int len = DIR == 0 ? nv : nh;
+  const int64_t n = (int64_t)nv * nh;
+  const int64_t step = (DIR == 0 ? 1 : (int64_t)nv) * B;  // elements between taps
+  const T l2 = (EPI == BAND_NORMAL || EPI == BAND_TRUERES) ? (T)lam2[col] : (T)0;
+  constexpr int U = sizeof(T) == 8 ? 8 : 16;  // taps in flight
+  DotAcc<T> dot;
+  // every lane of a warp runs the same number of steps (the vote below)
+  for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; p0 < n; p0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t p = p0 + lane;
+    const bool ok = p < n;
+    const int j = (n >> 31) == 0 ? (int)((unsigned)p / (unsigned)nv) : (int)(p / nv);
+    const int i = (int)(p - (int64_t)j * nv);
+    const int o = DIR == 0 ? i : j;
+    const T* __restrict__ x = in + ok * (p * B + col);
+    // taps inside the line: k0 <= k < k1
+    const int k0 = ok ? max(0, H - o) : 0, k1 = ok ? min(taps, len + H - o) : 0;
+    const bool edge = ok && bd.e != nullptr && (o < bd.nlo || o >= len - bd.nhi);
+    T acc = 0;
+    if (!__any_sync(0xffffffffu, edge || !ok || k0 > 0 || k1 < taps)) {
+      const T* xk = x - H * step;
+#pragma unroll U
+      for (int k = 0; k < taps; ++k) acc += bd.c[k] * xk[k * step];
+    } else if (!__any_sync(0xffffffffu, edge)) {
+      for (int kb = 0; kb < taps; kb += U) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int k = kb + u;  // c is zero beyond the taps (k1 <= taps)
+          acc += (k >= k0 && k < k1) ? bd.c[k < kBandMaxTaps ? k : 0] * x[(k - H) * step] : (T)0;
+        }
+      }
+    } else {
+      const int row = !edge ? bd.nlo + bd.nhi : (o < bd.nlo ? o : bd.nlo + o - (len - bd.nhi));
+      const T* __restrict__ e = bd.e + (int64_t)row * taps;
+      for (int kb = 0; kb < taps; kb += U) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int k = kb + u;
+          if (k >= k0 && k < k1) acc += e[k] * x[(k - H) * step];
+        }
+      }
+    }
+    if (!ok) continue;
+    if (EPI == BAND_STORE) {
+      out[p * B + col] = (TO)acc;
+    } else if (EPI == BAND_RESID2) {
+      const double e = to_d(acc) - bvec[p * B + col];
+      dot.add(e, e);
+    } else {
+      auto pv = [&](int64_t qq) { return P[qq * B + col]; };
+      const T kv = acc + l2 * fop.lap(p, i, j, pv);
+      if (EPI == BAND_NORMAL) {
+        out[p * B + col] = (TO)kv;
+        dot.add(P[p * B + col], kv);
+      } else {
+        const T rv = C[p * B + col] - kv;
+        out[p * B + col] = (TO)rv;
+        dot.add(rv, rv);
+      }
+    }
+  }
+  if (EPI != BAND_STORE) {
+    double dacc = dot.value();
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) dacc += __shfl_xor_sync(0xffffffffu, dacc, off);
+    if (lane == 0) sred[w] = dacc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double s = 0.0;
+      for (int k = 0; k < (int)blockDim.x / 32; ++k) s += sred[k];
       part[(int64_t)blockIdx.x * B + col] = s;
     }
   }
