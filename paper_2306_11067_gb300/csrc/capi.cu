@@ -71,6 +71,7 @@ struct Level {
   DevBuf<__half> hrows;
   DevBuf<float> hs;
   double glmax = 0.0, gamax = 0.0;
+  DevBuf<double> kr;       // FP64, one lambda per batch: the rows of K(lambda), 25 x n
   double hscale = 1.0;     // scale of the rows of the current lambda
 };
 
@@ -176,6 +177,7 @@ struct lcmg_ctx {
   double hw_scale = 1.0, hg_scale = 1.0;
   DevBuf<unsigned long long> hmax;
   bool h16_on = false;
+  bool k64_on = false;  // the coarse levels' kr hold the current batch's K(lambda)
   // hierarchy
   std::vector<Level> lev;
   bool hier_ok = false;
@@ -389,7 +391,7 @@ LevelView<double> view<double>(const lcmg_ctx& c, int k) {
   const Level& l = c.lev[k];
   v.nv = l.nv; v.nh = l.nh; v.n = l.n;
   if (k == 0) { v.fine = true; v.ws = c.ws.p; v.we = c.we.p; v.ga = c.diag.p; }
-  else { v.fine = false; v.cf = l.cf64.p; }
+  else { v.fine = false; v.cf = l.cf64.p; v.kr = c.k64_on ? l.kr.p : nullptr; }
   return v;
 }
 template <>
@@ -464,7 +466,7 @@ struct Batch {
   int tune_key() const { return 2 * B + (std::is_same<T, float>::value ? 1 : 0); }
 
   Batch(lcmg_ctx& c_, int B_) : c(c_), B(B_), s(c_.stream), nlev((int)c_.lev.size()) {
-    c.h16_on = false;
+    c.h16_on = c.k64_on = false;
     var_a = var_at = c.prm.spmv_variant;
     if (c.prm.spmv_variant_at) var_at = c.prm.spmv_variant_at;
     auto it = c.tuned.find(tune_key());
@@ -475,7 +477,7 @@ struct Batch {
     }
   }
 
-  ~Batch() { c.h16_on = false; }
+  ~Batch() { c.h16_on = c.k64_on = false; }
   Batch(const Batch&) = delete;
   Batch& operator=(const Batch&) = delete;
 
@@ -714,6 +716,14 @@ struct Batch {
         LCMG_LAUNCHED();
       }
       c.h16_on = true;
+    }
+    // FP64: the rows of K(lambda) of the levels the cycle relaxes on
+    c.k64_on = false;
+    if (std::is_same<T, double>::value && one_lam && c.prm.nu == 1 && vf_on()) {
+      for (int k = 1; k + 1 < nlev; ++k)
+        launch_rows64(c.lev[k].n, c.lev[k].gl.p, c.lev[k].ga.p, l2[0], c.lev[k].kr.need(kStencil * c.lev[k].n),
+                      c.maxblk, s);
+      c.k64_on = true;
     }
     for (int k = 0; k < nlev; ++k)
       launch_dinv<T>(view<T>(c, k), B, c.lam2.p, c.prm.smoother, c.prm.omega, tp(c.lw[k].dinv), c.maxblk, s);

@@ -24,6 +24,9 @@ struct LevelView {
   bool h16 = false;
   FineOpH fh{};
   CoarseOpH ch{};
+  // FP64, a batch whose columns share one lambda: the 25 coefficients of
+  // K(lambda) (coarse levels, [25][n]), or null
+  const T* kr = nullptr;
   FineOp<T> fine_op() const { return FineOp<T>{nv, nh, ws, we, ga}; }
   CoarseOp<T> coarse_op() const { return CoarseOp<T>{nv, nh, n, cf}; }
 };
@@ -61,6 +64,9 @@ int launch_vdown(const LevelView<T>& L, int B, const T* lam2, const T* dinv, con
 template <class T>
 int launch_vup(const LevelView<T>& L, int B, const T* lam2, const T* dinv, const T* r, const T* ec,
                const T* zpre, T* zout, double* part, int nu, cudaStream_t s);
+// kr = lam2 gl + ga, the rows of K(lambda) of a coarse level of n points
+void launch_rows64(int64_t n, const double* gl, const double* ga, double lam2, double* kr, int max_blocks,
+                   cudaStream_t s);
 // The finest level of the V(1,1) cycle for FP32 vectors (vfine.cuh): down
 // = z1 = D^{-1} r, residual and restriction (-> rc); up = z1 + P ec and one
 // sweep (-> zout, r.z partials into part when set).  D^{-1} from the stored

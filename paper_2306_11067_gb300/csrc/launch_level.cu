@@ -11,6 +11,7 @@
 #include "vtail.cuh"
 #include "vfine.cuh"
 #include "vfused.cuh"
+#include "vlevel64.cuh"
 
 namespace lcmg {
 
@@ -114,6 +115,70 @@ static int vup_one(const Op& op, int B, const T* lam2, const T* dinv, const T* r
   return g;
 }
 
+// FP64 with one sweep (vlevel64.cuh): f(integral_constant<tile side>, tiles
+// along i, tiles) with the side that leaves the fewest residual points on
+// the busiest SM.  A level of 512^2 points takes 8 x 8 coarse points (7
+// tiles of 18^2 on an SM), one of 32^2 takes 2 x 2 (64 tiles of 6^2 against 4 of
+// 18^2).  Measured on GB300 against 8 x 8 tiles with both parts of K read at
+// every point (down + up): 64 x 64 problem, its 32 x 32 level 11.5 + 9.7 ->
+// 5.7 + 5.6 us; 240 x 176, mean of three coarse levels 11.6 + 9.8 -> 5.8 +
+// 5.9 us; 1024 x 1024, mean of five 26.6 + 21.2 -> 14 + 10 us.
+template <class F>
+static int tiles64(int nvc, int nhc, int B, F&& f) {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    LCMG_CUDA(cudaGetDevice(&dev));
+    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  }
+  auto nt = [](int n, int tc) { return (n + tc - 1) / tc; };
+  int best = 8;
+  int64_t least = INT64_MAX;
+  for (int tc : {8, 4, 2}) {
+    const int64_t tiles = (int64_t)nt(nvc, tc) * nt(nhc, tc) * B;
+    const int64_t cost = (tiles + sms - 1) / sms * (2 * tc + 2) * (2 * tc + 2);
+    if (cost < least) {
+      least = cost;
+      best = tc;
+    }
+  }
+  const int ntx = nt(nvc, best), n = ntx * nt(nhc, best);
+  if (best == 8) return f(std::integral_constant<int, 8>{}, ntx, n);
+  if (best == 4) return f(std::integral_constant<int, 4>{}, ntx, n);
+  return f(std::integral_constant<int, 2>{}, ntx, n);
+}
+template <class Op>
+static int vdown64(const Op& op, int B, const double* lam2, const double* dinv, const double* r, double* zpre,
+                   double* rc, cudaStream_t s) {
+  return tiles64(op.nv / 2, op.nh / 2, B, [&](auto tc, int ntx, int nt) {
+    constexpr int TC = decltype(tc)::value;
+    auto k = k_vdown64<Op, TC>;
+    const int g = tile_grid(k, vt64_threads(TC), nt);
+    klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(vt64_threads(TC)), 0, s, op, B, lam2, dinv, r, zpre, rc, ntx, nt);
+    return g;
+  });
+}
+template <class Op>
+static int vup64(const Op& op, int B, const double* lam2, const double* dinv, const double* r, const double* ec,
+                 const double* zpre, double* zout, double* part, cudaStream_t s) {
+  return tiles64(op.nv / 2, op.nh / 2, B, [&](auto tc, int ntx, int nt) {
+    constexpr int TC = decltype(tc)::value;
+    auto k = k_vup64<Op, TC>;
+    const int g = tile_grid(k, vt64_threads(TC), nt);
+    klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(vt64_threads(TC)), 0, s, op, B, lam2, dinv, r, ec, zpre, zout,
+            ntx, nt, part);
+    return g;
+  });
+}
+
+void launch_rows64(int64_t n, const double* gl, const double* ga, double lam2, double* kr, int max_blocks,
+                   cudaStream_t s) {
+  const int64_t count = kStencil * n;
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>((count + kBlock - 1) / kBlock, max_blocks));
+  klaunch(k_rows64, dim3(g), dim3(kBlock), 0, s, count, gl, ga, lam2, kr);
+  LCMG_LAUNCHED();
+}
+
 // FP16 coarse levels with one sweep: the staged, double-buffered tile kernels
 static int vdown_h(const CoarseOpH& op, int B, const float* dinv, const float* r, float* zpre, float* rc, int ntx,
                    int ntiles, cudaStream_t s) {
@@ -150,7 +215,17 @@ int launch_vdown(const LevelView<T>& L, int B, const T* lam2, const T* dinv, con
       return g;
     }
   }
-  if (L.fine)
+  if constexpr (std::is_same<T, double>::value) {
+    if (nu == 1) {
+      g = L.fine ? vdown64(L.fine_op(), B, lam2, dinv, r, zpre, rc, s)
+          : L.kr ? vdown64(RowsOp64{L.nv, L.nh, L.n, L.kr}, B, lam2, dinv, r, zpre, rc, s)
+                 : vdown64(L.coarse_op(), B, lam2, dinv, r, zpre, rc, s);
+      LCMG_LAUNCHED();
+      return g;
+    }
+    g = L.fine ? vdown_one<FineOp<T>, T, 2>(L.fine_op(), B, lam2, dinv, r, zpre, rc, ntx, nt, s)
+               : vdown_one<CoarseOp<T>, T, 2>(L.coarse_op(), B, lam2, dinv, r, zpre, rc, ntx, nt, s);
+  } else if (L.fine)
     g = nu == 1 ? vdown_one<FineOp<T>, T, 1>(L.fine_op(), B, lam2, dinv, r, zpre, rc, ntx, nt, s)
                 : vdown_one<FineOp<T>, T, 2>(L.fine_op(), B, lam2, dinv, r, zpre, rc, ntx, nt, s);
   else
@@ -178,7 +253,17 @@ int launch_vup(const LevelView<T>& L, int B, const T* lam2, const T* dinv, const
       return g;
     }
   }
-  if (L.fine)
+  if constexpr (std::is_same<T, double>::value) {
+    if (nu == 1) {
+      g = L.fine ? vup64(L.fine_op(), B, lam2, dinv, r, ec, zpre, zout, part, s)
+          : L.kr ? vup64(RowsOp64{L.nv, L.nh, L.n, L.kr}, B, lam2, dinv, r, ec, zpre, zout, part, s)
+                 : vup64(L.coarse_op(), B, lam2, dinv, r, ec, zpre, zout, part, s);
+      LCMG_LAUNCHED();
+      return g;
+    }
+    g = L.fine ? vup_one<FineOp<T>, T, 2>(L.fine_op(), B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s)
+               : vup_one<CoarseOp<T>, T, 2>(L.coarse_op(), B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
+  } else if (L.fine)
     g = nu == 1 ? vup_one<FineOp<T>, T, 1>(L.fine_op(), B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s)
                 : vup_one<FineOp<T>, T, 2>(L.fine_op(), B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
   else
@@ -354,8 +439,8 @@ void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, i
   const double* src = M;
   for (int k = 0; k < nb; ++k) {  // the last step writes K
     double* dst = (nb - 1 - k) % 2 == 0 ? K : W;
-    klaunch(k_inverse_step, dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)B), dim3(4 * kInvTile * kInvTile), 0, s, n,
-            k, k == nb - 1 ? 1 : 0, src, dst, info);
+    klaunch(k_inverse_step, dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)B), dim3(4 * kInvTile * kInvTile), 0, s, n, k,
+            k == nb - 1 ? 1 : 0, src, dst, info);
     LCMG_LAUNCHED();
     src = dst;
   }
