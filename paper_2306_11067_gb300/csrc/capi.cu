@@ -759,7 +759,7 @@ struct Batch {
     int nb_rr;
     const bool alpha_fused = B == 1 && c.prm.alpha_fuse;
     if (alpha_fused) {  // alpha inside the update
-      nb_rr = launch_update_xr_alpha<T, T>(c.n, st, nb_pq, c.part_pq.p, P, Q, X, R, c.part_rr.p, c.maxblk, s);
+      nb_rr = launch_update_xr_alpha<T>(c.n, st, nb_pq, c.part_pq.p, P, Q, X, R, c.part_rr.p, c.maxblk, s);
     } else {
       klaunch(k_scalar_col_alpha, dim3(B), dim3(kColThreads), 0, s, B, nb_pq, c.part_pq.p, st);
       LCMG_LAUNCHED();

@@ -108,9 +108,9 @@ template <class T, class TX>
 int launch_update_xr(int64_t n, int B, const ColState& st, const T* p, const T* q, TX* x, T* r,
                      double* part, int max_blocks, cudaStream_t s);
 // one column: alpha from the p.q partials inside the update (no scalar kernel)
-template <class T, class TX>
+template <class T>
 int launch_update_xr_alpha(int64_t n, const ColState& st, int nb_pq, const double* pq_part, const T* p,
-                           const T* q, TX* x, T* r, double* part, int max_blocks, cudaStream_t s);
+                           const T* q, T* x, T* r, double* part, int max_blocks, cudaStream_t s);
 template <class T>
 void launch_update_p(int64_t n, int B, const ColState& st, const T* z, T* p, int max_blocks,
                      cudaStream_t s);

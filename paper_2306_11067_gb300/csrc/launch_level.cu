@@ -317,17 +317,18 @@ void launch_vtail(const TailLevelIn* levels, int nlev, const double* kinv, int n
   LCMG_LAUNCHED();
 }
 
-// Grid of the fused one-column updates: every block re-sums the partials of
-// the dot products it needs (FP64), so the grid stays at 4 blocks of 256
-// threads per SM (a full SM of resident warps streams the vectors)
-static int fused_update_grid(int64_t n, int max_blocks) {
+// Grid of the fused one-column updates: one 16-byte word per thread, at most
+// two blocks per SM (every block re-sums the partials of the dot products it
+// needs in FP64)
+static int fused_update_grid(int64_t words, int max_blocks) {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
     LCMG_CUDA(cudaGetDevice(&dev));
     LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   }
-  return std::min(grid_for(n, 1, max_blocks), std::max(1, 4 * sms));
+  const int64_t want = (words + kUpdThreads - 1) / kUpdThreads;
+  return (int)std::max<int64_t>(1, std::min(want, (int64_t)std::min(2 * sms, max_blocks)));
 }
 
 // Rows per strip of the row-streaming kernels: at most `most`, and few
@@ -463,11 +464,11 @@ int launch_update_xr(int64_t n, int B, const ColState& st, const T* p, const T* 
   return g;
 }
 
-template <class T, class TX>
+template <class T>
 int launch_update_xr_alpha(int64_t n, const ColState& st, int nb_pq, const double* pq_part, const T* p,
-                           const T* q, TX* x, T* r, double* part, int max_blocks, cudaStream_t s) {
-  const int g = fused_update_grid(n, max_blocks);
-  klaunch(k_update_xr_alpha<T, TX>, dim3(g), dim3(kBlock), 0, s, n, st, nb_pq, pq_part, p, q, x, r, part);
+                           const T* q, T* x, T* r, double* part, int max_blocks, cudaStream_t s) {
+  const int g = fused_update_grid(n / Pack<T>::W, max_blocks);
+  klaunch(k_update_xr_alpha<T>, dim3(g), dim3(kUpdThreads), 0, s, n, st, nb_pq, pq_part, p, q, x, r, part);
   LCMG_LAUNCHED();
   return g;
 }
@@ -476,8 +477,8 @@ template <class T>
 void launch_update_p_beta(int64_t n, const ColState& st, int nb_rr, const double* rr_part, int nb_rz,
                           const double* rz_part, int maxit, double rel_trigger, const T* z, T* p, int max_blocks,
                           cudaStream_t s) {
-  const int g = fused_update_grid(n, max_blocks);
-  klaunch(k_update_p_beta<T>, dim3(g), dim3(kBlock), 0, s, n, st, nb_rr, rr_part, nb_rz, rz_part, maxit, rel_trigger,
+  const int g = fused_update_grid(n / Pack<T>::W, max_blocks);
+  klaunch(k_update_p_beta<T>, dim3(g), dim3(kUpdThreads), 0, s, n, st, nb_rr, rr_part, nb_rz, rz_part, maxit, rel_trigger,
           z, p);
   LCMG_LAUNCHED();
 }
@@ -528,11 +529,9 @@ template int launch_update_xr<double, double>(int64_t, int, const ColState&, con
 template int launch_update_xr<float, float>(int64_t, int, const ColState&, const float*,
                                             const float*, float*, float*, double*, int,
                                             cudaStream_t);
-template int launch_update_xr_alpha<double, double>(int64_t, const ColState&, int, const double*,
-                                                    const double*, const double*, double*, double*,
-                                                    double*, int, cudaStream_t);
-template int launch_update_xr_alpha<float, float>(int64_t, const ColState&, int, const double*, const float*,
-                                                  const float*, float*, float*, double*, int,
-                                                  cudaStream_t);
+template int launch_update_xr_alpha<double>(int64_t, const ColState&, int, const double*, const double*,
+                                            const double*, double*, double*, double*, int, cudaStream_t);
+template int launch_update_xr_alpha<float>(int64_t, const ColState&, int, const double*, const float*, const float*,
+                                           float*, float*, double*, int, cudaStream_t);
 
 }  // namespace lcmg
