@@ -87,6 +87,7 @@ Band<T> make_band(const SepPass& p, const T* d_dev) {
   if (p.H < 0 || p.H > kBandMaxH) throw ArgError("band half-width out of range");
   Band<T> b{};
   b.H = p.H;
+  b.nch = (2 * p.H + 1 + kBandChunk - 1) / kBandChunk;
   for (int k = 0; k < kBandMaxTaps; ++k) b.c[k] = (k < (int)p.c.size()) ? (T)p.c[k] : (T)0;
   b.nlo = p.d.empty() ? 0 : p.nlo;
   b.nhi = p.d.empty() ? 0 : p.nhi;
@@ -95,113 +96,92 @@ Band<T> make_band(const SepPass& p, const T* d_dev) {
   return b;
 }
 
+// largest FP32 pass (points x columns) that runs with one output per thread
+constexpr int64_t kBandDirectMax = 256 * 256;
+
 // blocks of a banded pass resident at once on the current device
 template <class K>
-static int band_resident(K kern, int threads) {
+static int band_resident(K kern, size_t smem) {
   static std::mutex mu;
-  static std::map<std::pair<const void*, int>, int> cache;
+  static std::map<std::pair<const void*, std::pair<int, size_t>>, int> cache;
   int dev = 0;
   LCMG_CUDA(cudaGetDevice(&dev));
-  const auto key = std::make_pair(reinterpret_cast<const void*>(kern), dev);
+  const auto key = std::make_pair(reinterpret_cast<const void*>(kern), std::make_pair(dev, smem));
   std::lock_guard<std::mutex> lock(mu);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
   int nb = 0, sms = 0;
-  LCMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, 0));
+  LCMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kBandThreads, smem));
   LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (nb < 1) throw CudaError("banded pass does not fit on an SM");
   cache[key] = nb * sms;
   return nb * sms;
 }
 
-static int clamp_blocks(int64_t want, int64_t most) { return (int)std::max<int64_t>(1, std::min(want, most)); }
-
-// FP32, large images: the tap count rounded up to a compiled one
-template <class F>
-static int by_taps(int taps, F&& f) {
-  if (taps <= 17) return f(std::integral_constant<int, 17>{});
-  if (taps <= 25) return f(std::integral_constant<int, 25>{});
-  if (taps <= 37) return f(std::integral_constant<int, 37>{});
-  if (taps <= 49) return f(std::integral_constant<int, 49>{});
-  if (taps <= 61) return f(std::integral_constant<int, 61>{});
-  return f(std::integral_constant<int, 65>{});
-}
-// everything in 16-byte words: one column, lines of a multiple of 4 points
-static bool band_wide(int nv, int B) { return B == 1 && nv % 4 == 0; }
-
-static int band_line(int nv, int nh, int B, const Band<float>& bd, const float* in, float* out, int max_blocks,
-                     cudaStream_t s) {
-  return by_taps(2 * bd.H + 1, [&](auto taps) {
-    constexpr int TAPS = decltype(taps)::value;
-    auto k = band_wide(nv, B) ? k_band_line<TAPS, true> : k_band_line<TAPS, false>;
-    const int64_t tasks = (int64_t)((nv + kLineSeg - 1) / kLineSeg) * nh * B;
-    const int blocks = clamp_blocks((tasks + kLineWarps - 1) / kLineWarps, max_blocks);
-    klaunch(k, dim3((unsigned)blocks), dim3(32 * kLineWarps), 0, s, nv, nh, B, bd, in, out);
-    LCMG_LAUNCHED();
-    return blocks;
-  });
-}
-static int band_rows(int nv, int nh, int B, const Band<float>& bd, const float* in, float* out,
-                     const FineOp<float>& fop, const float* P, const double* lam2, double* part, int max_blocks,
-                     cudaStream_t s) {
-  return by_taps(2 * bd.H + 1, [&](auto taps) {
-    constexpr int TAPS = decltype(taps)::value;
-    auto k = band_wide(nv, B) ? k_band_rows<TAPS, true> : k_band_rows<TAPS, false>;
-    const int64_t tiles = (int64_t)((nv + 31) / 32) * ((nh + kRowTile - 1) / kRowTile);
-    const int blocks = clamp_blocks(tiles, max_blocks);
-    klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(32 * kRowWarps), sizeof(float) * rows_floats(TAPS), s, nv, nh,
-            B, bd, in, out, fop, P, lam2, part);
-    LCMG_LAUNCHED();
-    return blocks;
-  });
-}
-
-// opt k_band_rows into its shared memory on the current device (outside
-// stream capture)
-void prepare_band() {
-  for (int taps : {17, 25, 37, 49, 61, 65})
-    by_taps(taps, [&](auto t) {
-      constexpr int TAPS = decltype(t)::value;
-      const int bytes = (int)sizeof(float) * rows_floats(TAPS);
-      LCMG_CUDA(cudaFuncSetAttribute(k_band_rows<TAPS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      LCMG_CUDA(cudaFuncSetAttribute(k_band_rows<TAPS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      return 0;
-    });
+template <class T, class TO, int DIR, int EPI, int TAPS>
+static int band_go(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
+                   const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s) {
+  auto k = k_band<T, TO, DIR, EPI, TAPS>;
+  const size_t smem = band_smem_bytes<T>(bd.nch);
+  const int len = DIR == 0 ? nv : nh, lines = DIR == 0 ? nh : nv;
+  const int64_t tiles = (int64_t)((len + kBandSeg - 1) / kBandSeg) * ((lines + kBandLines - 1) / kBandLines);
+  int64_t blocks = std::min<int64_t>(tiles, band_resident(k, smem));
+  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, max_blocks));
+  klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(kBandThreads), smem, s, nv, nh, B, bd, in, out, fop, P, C,
+          lam2, bvec, part);
+  LCMG_LAUNCHED();
+  return (int)blocks;
 }
 
 template <class T, class TO, int DIR, int EPI>
-static int band_direct(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop,
-                       const T* P, const T* C, const double* lam2, const double* bvec, double* part, int max_blocks,
-                       cudaStream_t s) {
+static int band_direct_go(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop,
+                          const T* P, const T* C, const double* lam2, const double* bvec, double* part,
+                          int max_blocks, cudaStream_t s) {
   auto k = k_band_direct<T, TO, DIR, EPI>;
   const int64_t n = (int64_t)nv * nh;
   // small images in blocks of two warps, so that they spread over more SMs
   const int threads = n <= 64 * 1024 ? 64 : kBandThreads;
-  const int blocks = clamp_blocks((n + threads - 1) / threads, std::min(max_blocks, band_resident(k, kBandThreads)));
+  int64_t blocks = std::min<int64_t>((n + threads - 1) / threads, band_resident(k, 0));
+  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, max_blocks));
   klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(threads), 0, s, nv, nh, B, bd, in, out, fop, P, C, lam2, bvec,
           part);
   LCMG_LAUNCHED();
-  return blocks;
+  return (int)blocks;
 }
 
-// FP32 passes of at most this many points x columns run with one output per
-// thread: the other kernels give a thread 8 or 16 outputs, so that below it
-// part of the GPU has none.  Measured on GB300: DIRECT32.
-constexpr int64_t kBandDirectMax = 512 * 512;
-
+// FP64, and FP32 images whose tiles would leave most of the GPU idle: one
+// output per thread.  FP32 otherwise: staged tiles, with the tap count of
+// the A^T A passes of radii 4, 9 and 15 (17, 37 and 61 taps) compiled in,
+// every other pass with the chunked loop.
 template <class T, class TO, int DIR, int EPI>
 int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
                 const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s) {
-  if constexpr (std::is_same<T, float>::value) {
-    if ((int64_t)nv * nh * B > kBandDirectMax) {
-      static_assert((DIR == 0 && EPI == BAND_STORE) || (DIR == 1 && EPI == BAND_NORMAL), "the FP32 passes of A^T A");
-      if constexpr (DIR == 0)
-        return band_line(nv, nh, B, bd, in, out, max_blocks, s);
-      else
-        return band_rows(nv, nh, B, bd, in, out, fop, P, lam2, part, max_blocks, s);
+  if constexpr (std::is_same<T, double>::value) {
+    return band_direct_go<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+  } else {
+    if ((int64_t)nv * nh * B <= kBandDirectMax)
+      return band_direct_go<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+    switch (2 * bd.H + 1) {
+      case 17: return band_go<T, TO, DIR, EPI, 17>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+      case 37: return band_go<T, TO, DIR, EPI, 37>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+      case 61: return band_go<T, TO, DIR, EPI, 61>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+      default: return band_go<T, TO, DIR, EPI, 0>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
     }
   }
-  return band_direct<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+}
+
+template <class T, class TO, int DIR, int EPI>
+static void band_optin() {
+  const int bytes = (int)band_smem_bytes<T>((2 * kBandMaxH + 1 + kBandChunk - 1) / kBandChunk);
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 17>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 37>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 61>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+}
+
+void prepare_band() {
+  band_optin<float, float, 0, BAND_STORE>();
+  band_optin<float, float, 1, BAND_NORMAL>();
 }
 
 void launch_sep_diag(int nv, int nh, const double* dv, const double* dh, double* diag, int max_blocks,
