@@ -29,6 +29,13 @@ __device__ __forceinline__ T pw1(int a, int I, int nc) {
   return T(0);
 }
 
+// sum of v over a warp, in every lane
+__device__ __forceinline__ double warp_sum64(double v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
 // Compensated dot product in the working precision (Ogita, Rump and Oishi,
 // "Accurate sum and dot product", 2005, Algorithm Dot2): each product is
 // split exactly into p + e with one FMA, the running sum is kept exact to
@@ -47,6 +54,7 @@ struct Dot2 {
     s = t;
   }
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+  __device__ __forceinline__ double warp_sum() const { return warp_sum64(value()); }
 };
 
 // A thread's dot-product accumulator: FP64 for FP64 vectors, Dot2 for FP32
@@ -55,6 +63,7 @@ struct DotAcc {
   double s = 0.0;
   __device__ __forceinline__ void add(double a, double b) { s += a * b; }
   __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ double warp_sum() const { return warp_sum64(s); }
 };
 template <>
 struct DotAcc<float> : Dot2 {};

@@ -149,7 +149,7 @@ Band<T> make_band(const SepPass& p, const T* d_dev);
 template <class T, class TO, int DIR, int EPI>
 int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
                 const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s);
-// opt every k_band instantiation into its shared memory on the current
+// opt the banded kernels into their shared memory on the current
 // device (outside stream capture)
 void prepare_band();
 // diag(A^T A)_p = dv[i] dh[j]

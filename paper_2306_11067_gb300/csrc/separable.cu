@@ -1,6 +1,6 @@
 // Host side of the separable blur operator: the coefficient sets of the
 // banded 1-D passes (built in FP64 from the 1-D PSF factors) and the
-// launchers of k_band.
+// launchers of its kernels.
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -96,9 +96,6 @@ Band<T> make_band(const SepPass& p, const T* d_dev) {
   return b;
 }
 
-// largest FP32 pass (points x columns) that runs with one output per thread
-constexpr int64_t kBandDirectMax = 256 * 256;
-
 // blocks of a banded pass resident at once on the current device
 template <class K>
 static int band_resident(K kern, size_t smem) {
@@ -118,70 +115,132 @@ static int band_resident(K kern, size_t smem) {
   return nb * sms;
 }
 
+static int clamp_blocks(int64_t want, int64_t most) { return (int)std::max<int64_t>(1, std::min(want, most)); }
+
 template <class T, class TO, int DIR, int EPI, int TAPS>
-static int band_go(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
+static int band_tiles(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
                    const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s) {
   auto k = k_band<T, TO, DIR, EPI, TAPS>;
   const size_t smem = band_smem_bytes<T>(bd.nch);
   const int len = DIR == 0 ? nv : nh, lines = DIR == 0 ? nh : nv;
   const int64_t tiles = (int64_t)((len + kBandSeg - 1) / kBandSeg) * ((lines + kBandLines - 1) / kBandLines);
-  int64_t blocks = std::min<int64_t>(tiles, band_resident(k, smem));
-  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, max_blocks));
+  const int blocks = clamp_blocks(tiles, std::min(max_blocks, band_resident(k, smem)));
   klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(kBandThreads), smem, s, nv, nh, B, bd, in, out, fop, P, C,
           lam2, bvec, part);
   LCMG_LAUNCHED();
-  return (int)blocks;
+  return blocks;
+}
+
+// k_band_line and k_band_rows: the tap count rounded up to a compiled one
+template <class F>
+static int by_taps(int taps, F&& f) {
+  if (taps <= 17) return f(std::integral_constant<int, 17>{});
+  if (taps <= 25) return f(std::integral_constant<int, 25>{});
+  if (taps <= 37) return f(std::integral_constant<int, 37>{});
+  if (taps <= 49) return f(std::integral_constant<int, 49>{});
+  if (taps <= 61) return f(std::integral_constant<int, 61>{});
+  return f(std::integral_constant<int, 65>{});
+}
+
+static int band_line(int nv, int nh, const Band<float>& bd, const float* in, float* out, int max_blocks,
+                     cudaStream_t s) {
+  return by_taps(2 * bd.H + 1, [&](auto taps) {
+    constexpr int TAPS = decltype(taps)::value;
+    const int64_t tasks = (int64_t)((nv + kLineSeg - 1) / kLineSeg) * nh;
+    const int blocks = clamp_blocks((tasks + kLineWarps - 1) / kLineWarps, max_blocks);
+    klaunch(k_band_line<TAPS>, dim3((unsigned)blocks), dim3(32 * kLineWarps), 0, s, nv, nh, bd, in, out);
+    LCMG_LAUNCHED();
+    return blocks;
+  });
+}
+static int band_rows(int nv, int nh, const Band<float>& bd, const float* in, float* out,
+                     const FineOp<float>& fop, const float* P, const double* lam2, double* part, int max_blocks,
+                     cudaStream_t s) {
+  return by_taps(2 * bd.H + 1, [&](auto taps) {
+    constexpr int TAPS = decltype(taps)::value;
+    const int64_t tiles = (int64_t)((nv + 31) / 32) * ((nh + kRowTile - 1) / kRowTile);
+    const int blocks = clamp_blocks(tiles, max_blocks);
+    klaunch(k_band_rows<TAPS>, dim3((unsigned)blocks), dim3(32 * kRowWarps), sizeof(float) * rows_floats(TAPS), s, nv,
+            nh, bd, in, out, fop, P, lam2, part);
+    LCMG_LAUNCHED();
+    return blocks;
+  });
+}
+
+// opt k_band and k_band_rows into their shared memory on the current device
+// (outside stream capture)
+template <int DIR, int EPI, int TAPS>
+static void band_optin() {
+  const int bytes = (int)band_smem_bytes<float>((2 * kBandMaxH + 1 + kBandChunk - 1) / kBandChunk);
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<float, float, DIR, EPI, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+}
+template <int DIR, int EPI>
+static void band_optin_taps() {
+  band_optin<DIR, EPI, 0>();
+  band_optin<DIR, EPI, 17>();
+  band_optin<DIR, EPI, 37>();
+  band_optin<DIR, EPI, 61>();
+}
+void prepare_band() {
+  for (int taps : {17, 25, 37, 49, 61, 65})
+    by_taps(taps, [&](auto t) {
+      constexpr int TAPS = decltype(t)::value;
+      LCMG_CUDA(cudaFuncSetAttribute(k_band_rows<TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(float) * rows_floats(TAPS)));
+      return 0;
+    });
+  band_optin_taps<0, BAND_STORE>();
+  band_optin_taps<1, BAND_NORMAL>();
 }
 
 template <class T, class TO, int DIR, int EPI>
-static int band_direct_go(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop,
-                          const T* P, const T* C, const double* lam2, const double* bvec, double* part,
-                          int max_blocks, cudaStream_t s) {
+static int band_direct(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop,
+                       const T* P, const T* C, const double* lam2, const double* bvec, double* part, int max_blocks,
+                       cudaStream_t s) {
   auto k = k_band_direct<T, TO, DIR, EPI>;
   const int64_t n = (int64_t)nv * nh;
   // small images in blocks of two warps, so that they spread over more SMs
   const int threads = n <= 64 * 1024 ? 64 : kBandThreads;
-  int64_t blocks = std::min<int64_t>((n + threads - 1) / threads, band_resident(k, 0));
-  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, max_blocks));
+  const int blocks = clamp_blocks((n + threads - 1) / threads, std::min(max_blocks, band_resident(k, 0)));
   klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(threads), 0, s, nv, nh, B, bd, in, out, fop, P, C, lam2, bvec,
           part);
   LCMG_LAUNCHED();
-  return (int)blocks;
+  return blocks;
 }
 
-// FP64, and FP32 images whose tiles would leave most of the GPU idle: one
-// output per thread.  FP32 otherwise: staged tiles, with the tap count of
-// the A^T A passes of radii 4, 9 and 15 (17, 37 and 61 taps) compiled in,
-// every other pass with the chunked loop.
+// FP32 passes of at most this many points (x columns) run with one output per
+// thread: the other kernels give a thread 16, so that below it part of the GPU
+// has none.  Measured on GB300, both passes of A^T A, one column: 384 x 384,
+// 61 taps 20.6 us against 22.6 in k_band_line + k_band_rows, 448 x 448 24.6
+// against 22.6, 512 x 512 28.8 against 24.6; 37 taps 16.5 / 19.7, 21.4 / 20.5,
+// 22.6 / 20.5.
+constexpr int64_t kBandDirectMax = 440 * 440;
+constexpr int64_t kBandDirectMaxTiles = 256 * 256;  // ... where the alternative is k_band
+
 template <class T, class TO, int DIR, int EPI>
 int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
                 const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s) {
-  if constexpr (std::is_same<T, double>::value) {
-    return band_direct_go<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-  } else {
-    if ((int64_t)nv * nh * B <= kBandDirectMax)
-      return band_direct_go<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-    switch (2 * bd.H + 1) {
-      case 17: return band_go<T, TO, DIR, EPI, 17>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-      case 37: return band_go<T, TO, DIR, EPI, 37>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-      case 61: return band_go<T, TO, DIR, EPI, 61>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-      default: return band_go<T, TO, DIR, EPI, 0>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+  if constexpr (std::is_same<T, float>::value) {
+    static_assert((DIR == 0 && EPI == BAND_STORE) || (DIR == 1 && EPI == BAND_NORMAL), "the FP32 passes of A^T A");
+    const int64_t work = (int64_t)nv * nh * B;
+    if (B == 1 && nv % 4 == 0) {  // 16-byte words (every vector of a solve starts on such a boundary)
+      if (work > kBandDirectMax) {
+        if constexpr (DIR == 0)
+          return band_line(nv, nh, bd, in, out, max_blocks, s);
+        else
+          return band_rows(nv, nh, bd, in, out, fop, P, lam2, part, max_blocks, s);
+      }
+    } else if (work > kBandDirectMaxTiles) {
+      // the tap counts of the A^T A passes of radii 4, 9 and 15 compiled in
+      switch (2 * bd.H + 1) {
+        case 17: return band_tiles<T, TO, DIR, EPI, 17>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+        case 37: return band_tiles<T, TO, DIR, EPI, 37>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+        case 61: return band_tiles<T, TO, DIR, EPI, 61>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+        default: return band_tiles<T, TO, DIR, EPI, 0>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
+      }
     }
   }
-}
-
-template <class T, class TO, int DIR, int EPI>
-static void band_optin() {
-  const int bytes = (int)band_smem_bytes<T>((2 * kBandMaxH + 1 + kBandChunk - 1) / kBandChunk);
-  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 17>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 37>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, TO, DIR, EPI, 61>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-}
-
-void prepare_band() {
-  band_optin<float, float, 0, BAND_STORE>();
-  band_optin<float, float, 1, BAND_NORMAL>();
+  return band_direct<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
 }
 
 void launch_sep_diag(int nv, int nh, const double* dv, const double* dh, double* diag, int max_blocks,
