@@ -69,7 +69,8 @@ struct Level {
   // FP16 smoother data (levels >= 1): per-lambda rows of K's off-diagonals,
   // the row sums of G_A, and the largest off-diagonal |G_L|, |G_A| (scales)
   DevBuf<__half> hrows;
-  DevBuf<float> hs;
+  DevBuf<float> hs;        // row sums of G_A
+  DevBuf<float> hc;        // diagonals of the current lambda's rows, in their scale
   double glmax = 0.0, gamax = 0.0;
   DevBuf<double> kr;       // FP64, one lambda per batch: the rows of K(lambda), 25 x n
   double hscale = 1.0;     // scale of the rows of the current lambda
@@ -319,7 +320,8 @@ static void build_half(lcmg_ctx& c) {
     LCMG_LAUNCHED();
     klaunch(k_rowsum25, dim3(gk), dim3(kBlock), 0, c.stream, g.n, (const double*)g.ga.p, g.hs.need(g.n));
     LCMG_LAUNCHED();
-    g.hrows.need((size_t)kCompactOff * g.n);
+    g.hrows.need((size_t)CoarseOpH::size(g.nv, g.nh));
+    g.hc.need(g.n);
   }
   std::vector<unsigned long long> hm(2 * L + 2);
   copy_sync(c.stream, hm.data(), mx, sizeof(unsigned long long) * hm.size(), cudaMemcpyDeviceToHost);
@@ -404,7 +406,7 @@ LevelView<float> view<float>(const lcmg_ctx& c, int k) {
   if (c.h16_on) {
     v.h16 = true;
     v.fh = FineOpH{l.nv, l.nh, c.h_ws.p, c.h_we.p, c.h_ga.p, (float)(1.0 / c.hw_scale), (float)(1.0 / c.hg_scale)};
-    v.ch = CoarseOpH{l.nv, l.nh, l.n, reinterpret_cast<const uint4*>(l.hrows.p), l.hs.p, (float)(1.0 / l.hscale)};
+    v.ch = CoarseOpH{l.nv, l.nh, l.n, l.hrows.p, l.hc.p, (float)(1.0 / l.hscale)};
   }
   return v;
 }
@@ -572,13 +574,14 @@ struct Batch {
     for (int k = 0; k + 1 < nlev; ++k) {
       const int64_t nk = c.lev[k].n;
       int64_t coef = k == 0 ? 3 * sT : (int64_t)kCoefStride * sT;
-      if (c.h16_on) coef = k == 0 ? 3 * 2 : kCompactOff * 2 + 4;  // FP16 rows (+ FP32 row sum)
+      if (c.h16_on) coef = k == 0 ? 3 * 2 : kCompactOff * 2 + 4;  // FP16 rows (+ FP32 diagonal)
       if (k == 0 && fine_v11()) {
         // r twice, r_c and e_c (a quarter each), z once; no pre-smoothed z, no D^{-1}
         bytes += (nk * 7 / 2) * sT * B + 2 * coef * nk;
         continue;
       }
-      bytes += (nk * 15 / 2) * sT * B + 2 * coef * nk;
+      // FP16 coarse levels with one sweep form the pre-smoothed z in both kernels
+      bytes += (c.h16_on && c.prm.nu == 1 ? nk * 11 / 2 : nk * 15 / 2) * sT * B + 2 * coef * nk;
     }
     const int64_t nc = c.lev[nlev - 1].n;
     bytes += (nc * nc * 8 + 2 * nc * sT) * B;
@@ -710,9 +713,9 @@ struct Batch {
       for (int k = 1; k < nlev; ++k) {
         Level& g = c.lev[k];
         g.hscale = half_scale(l2[0] * g.glmax + g.gamax);
-        const int gg = (int)std::min<int64_t>((kCompactOff * g.n + kBlock - 1) / kBlock, c.maxblk);
-        klaunch(k_compact_rows, dim3(gg), dim3(kBlock), 0, s, g.n, (const double*)g.gl.p, (const double*)g.ga.p,
-                l2[0], g.hscale, g.hrows.p);
+        const int gg = (int)std::min<int64_t>((g.n + kBlock - 1) / kBlock, c.maxblk);
+        klaunch(k_compact_rows, dim3(gg), dim3(kBlock), 0, s, g.nv, g.nh, g.n, (const double*)g.gl.p,
+                (const double*)g.ga.p, l2[0], g.hscale, (const float*)g.hs.p, g.hrows.p, g.hc.p);
         LCMG_LAUNCHED();
       }
       c.h16_on = true;

@@ -16,11 +16,11 @@
 //    diagonal) with every weight rounded to 11 significant bits;
 //  * coarse level k: per lambda, the 24 off-diagonal coefficients of
 //    K_k(lam) = lam^2 G_L^k + G_A^k, FP16 (48 bytes per point against 256
-//    for the FP32 rows of both parts), and the row sums s = G_A^k 1 in FP32
-//    (lambda-independent: the rows of G_L^k sum to zero); the diagonal is
-//    s_p minus the sum of the stored off-diagonals, so K^ 1 = G_A 1 exactly
-//    and the rounding perturbs K by a zero-row-sum (Laplacian-like) term of
-//    relative size 2^-11 that keeps it positive definite.
+//    for the FP32 rows of both parts), and the diagonal in FP32: the row sum
+//    s_p = (G_A^k 1)_p (the rows of G_L^k sum to zero) minus the sum of the
+//    stored off-diagonals, so K^ 1 = G_A 1 exactly and the rounding perturbs
+//    K by a zero-row-sum (Laplacian-like) term of relative size 2^-11 that
+//    keeps it positive definite.
 //
 // The coarsest level keeps its exact FP64 factorisation.  Tested against
 // the oracle's model of the same storage (oracle.multigrid, storage="fp16").
@@ -95,71 +95,37 @@ struct FineOpH {
   }
 };
 
-// coarse level in FP16: row p holds the off-diagonal coefficients of
-// K(lam) for the offsets o = (di+2) + 5 (dj+2) in increasing o, o = 12 left
-// out, scaled by 2^e; the diagonal is s[p] minus their sum
+// Coarse level in FP16: the off-diagonal coefficients of K(lam) for the
+// offsets o = (di+2) + 5 (dj+2) in increasing o, o = 12 left out, scaled by
+// 2^e, and per point the diagonal in the same units (the row sum of G_A
+// minus the stored off-diagonals).  The coefficients of 64 points of a grid
+// row lie together, [row j][block of 64 along i][24][64], so a warp reads
+// one coefficient of 64 points as one 128-byte line, the 24 of them at
+// fixed distances from one address.
 struct CoarseOpH {
   int nv, nh;
   int64_t n;
-  const uint4* __restrict__ rows;  // 3 x 16 bytes per point
-  const float* __restrict__ s;     // row sums of G_A
+  const __half* __restrict__ rows;
+  const float* __restrict__ c;     // diagonals x 2^e
   float sc;                        // 2^-e
   static constexpr int kRadius = 2;
 
+  __host__ __device__ static int64_t blocks(int nv) { return (nv + 63) / 64; }
+  // elements of `rows`
+  __host__ __device__ static int64_t size(int nv, int nh) { return blocks(nv) * nh * (24 * 64); }
+  // the first coefficient of point (i, j); coefficient h follows at + 64 h
+  __device__ __forceinline__ const __half* at(int i, int j) const {
+    return rows + ((int64_t)j * blocks(nv) + (i >> 6)) * (24 * 64) + (i & 63);
+  }
+
   // k[o] of K(lam) for o < 25 (lam2 is already in the stored rows)
   __device__ __forceinline__ void coefs(int64_t p, float, float (&k)[28]) const {
-    decode(rows[3 * p], rows[3 * p + 1], rows[3 * p + 2], s[p], k);
-  }
-  // the same from a row's three 16-byte words and its row sum
-  __device__ __forceinline__ void decode(const uint4 q0, const uint4 q1, const uint4 q2, const float sp,
-                                        float (&k)[28]) const {
-    const uint32_t w[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
-    float off[kCompactOff];
+    const int j = (int)(p / nv), i = (int)(p - (int64_t)j * nv);
+    const __half* q = at(i, j);
 #pragma unroll
-    for (int h = 0; h < 12; ++h) {
-      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[h]));
-      off[2 * h] = f.x * sc;
-      off[2 * h + 1] = f.y * sc;
-    }
-    float sum = 0;
-#pragma unroll
-    for (int o = 0; o < kCompactOff; ++o) sum += off[o];
-#pragma unroll
-    for (int o = 0; o < 12; ++o) k[o] = off[o];
-    k[12] = sp - sum;
-#pragma unroll
-    for (int o = 13; o < 25; ++o) k[o] = off[o - 1];
+    for (int h = 0; h < kCompactOff; ++h) k[h < 12 ? h : h + 1] = __half2float(q[64 * h]) * sc;
+    k[12] = c[p] * sc;
     k[25] = k[26] = k[27] = 0;
-  }
-  // (K v)_p from the point's three row words and row sum, every one of the
-  // 25 terms taken (the caller's v is zero outside the grid, so the terms
-  // apply_k leaves out add nothing).  The products are formed with the
-  // stored FP16 values and the sum scaled by sc at the end: sc and its
-  // inverse are powers of two, so every product and partial sum is the one
-  // apply_k forms, times 2^e exactly, and the result is the same float.
-  template <class F>
-  __device__ __forceinline__ float apply_rows(const uint4 q0, const uint4 q1, const uint4 q2, const float sp,
-                                              float inv_sc, F v) const {
-    const uint32_t w[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
-    float off[kCompactOff];
-#pragma unroll
-    for (int h = 0; h < 12; ++h) {
-      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[h]));
-      off[2 * h] = f.x;
-      off[2 * h + 1] = f.y;
-    }
-    float sum = 0;
-#pragma unroll
-    for (int o = 0; o < kCompactOff; ++o) sum += off[o];
-    const float center = sp * inv_sc - sum;
-    float acc = 0;
-#pragma unroll
-    for (int o = 0; o < 25; ++o) {
-      const int dj = o / 5 - 2, di = o % 5 - 2;
-      const float k = o < 12 ? off[o] : (o == 12 ? center : off[o - 1]);
-      acc += k * v(di, dj);
-    }
-    return acc * sc;
   }
   template <class F>
   __device__ __forceinline__ float apply_k(const float (&k)[28], int i, int j, F v) const {
@@ -241,16 +207,27 @@ static __global__ void k_maxabs(int64_t n, const double* __restrict__ v, int ste
   if ((threadIdx.x & 31) == 0) atomicMax(mx, (unsigned long long)__double_as_longlong(m));
 }
 
-// the coarse rows of K(lam) = lam2 G_L + G_A (off-diagonals, FP16, x scale)
-static __global__ void k_compact_rows(int64_t n, const double* __restrict__ gl, const double* __restrict__ ga,
-                                      double lam2, double scale, __half* __restrict__ rows) {
-  for (int64_t t = (int64_t)blockIdx.x * kBlock + threadIdx.x; t < n * kCompactOff;
-       t += (int64_t)gridDim.x * kBlock) {
-    const int64_t p = t / kCompactOff;
-    const int h = (int)(t - p * kCompactOff);
-    const int o = h < 12 ? h : h + 1;
-    const double k = lam2 * gl[(int64_t)o * n + p] + ga[(int64_t)o * n + p];
-    rows[t] = __double2half(k * scale);
+// The rows of K(lam) = lam2 G_L + G_A in FP16 (x scale, a power of two) and
+// their diagonals: s the row sums of G_A.  One thread per point, so that
+// every access runs along the points; it was one thread per coefficient with
+// the 24 of a point together (48 bytes apart in every read of G_L and G_A).
+static __global__ void __launch_bounds__(kBlock)
+    k_compact_rows(int nv, int nh, int64_t n, const double* __restrict__ gl, const double* __restrict__ ga, double lam2,
+                   double scale, const float* __restrict__ s, __half* __restrict__ rows, float* __restrict__ c) {
+  const float fscale = (float)scale;
+  for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n; p += (int64_t)gridDim.x * kBlock) {
+    const int j = (int)(p / nv), i = (int)(p - (int64_t)j * nv);
+    __half* q = rows + ((int64_t)j * CoarseOpH::blocks(nv) + (i >> 6)) * (24 * 64) + (i & 63);
+    float sum = 0.f;
+#pragma unroll 8
+    for (int h = 0; h < kCompactOff; ++h) {
+      const int o = h < 12 ? h : h + 1;
+      const double k = lam2 * gl[(int64_t)o * n + p] + ga[(int64_t)o * n + p];
+      const __half v = __double2half(k * scale);
+      q[64 * h] = v;
+      sum += __half2float(v);
+    }
+    c[p] = s[p] * fscale - sum;
   }
 }
 

@@ -179,22 +179,42 @@ void launch_rows64(int64_t n, const double* gl, const double* ga, double lam2, d
   LCMG_LAUNCHED();
 }
 
-// FP16 coarse levels with one sweep: the staged, double-buffered tile kernels
-static int vdown_h(const CoarseOpH& op, int B, const float* dinv, const float* r, float* zpre, float* rc, int ntx,
-                   int ntiles, cudaStream_t s) {
-  const size_t smem = 2 * sizeof(VcDownStage);
-  const int g = tile_grid(k_vdown_h, kVcThreads, ntiles, smem);
-  klaunch(k_vdown_h, dim3((unsigned)g, (unsigned)B), dim3(kVcThreads), smem, s, op, B, dinv, r, zpre, rc, ntx,
-          ntiles);
+// FP16 coarse levels with one sweep (vcoarse.cuh): coarse rows per strip, so
+// that the strips make kVcWarps warps per SM (of at most 16 rows; a strip
+// reads two residual rows more than it produces).  Measured on GB300 at
+// 1024^2 points with 8, 16 and 24 warps: down 23.7, 18.4, 22.1 us.
+static int coarse_strip(int nsi, int nhc, int B) {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    LCMG_CUDA(cudaGetDevice(&dev));
+    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  }
+  const int64_t per_col = std::max<int64_t>(1, ((int64_t)sms * kVcWarps) / ((int64_t)nsi * B));
+  return std::max(1, std::min(16, (int)((nhc + per_col - 1) / per_col)));
+}
+template <class K, class... A>
+static int strips_h(K k, int nsi, int crows, const CoarseOpH& op, int B, cudaStream_t s, A... args) {
+  const int nst = nsi * ((op.nh / 2 + crows - 1) / crows), wpb = kVcThreads / 32;
+  const int g = (nst + wpb - 1) / wpb;
+  klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(kVcThreads), 0, s, op, B, args..., nsi, nst, crows);
   return g;
 }
-static int vup_h(const CoarseOpH& op, int B, const float* dinv, const float* r, const float* ec, const float* zpre,
-                 float* zout, double* part, int ntx, int ntiles, cudaStream_t s) {
-  const size_t smem = 2 * sizeof(VcUpStage);
-  const int g = tile_grid(k_vup_h, kVcThreads, ntiles, smem);
-  klaunch(k_vup_h, dim3((unsigned)g, (unsigned)B), dim3(kVcThreads), smem, s, op, B, dinv, r, ec, zpre, zout, ntx,
-          ntiles, part);
-  return g;
+static int vdown_h(const CoarseOpH& op, int B, const float* dinv, const float* r, float* rc, cudaStream_t s) {
+  const int nsi = (op.nv / 2 + kVcDownCols - 1) / kVcDownCols, g = nsi * (op.nh / 2);
+  const int crows = coarse_strip(nsi, op.nh / 2, B);
+  if (crows == 1) {  // levels of 256^2 points (columns included) and below
+    klaunch(B == 1 ? k_vdown_h1<true> : k_vdown_h1<false>, dim3((unsigned)g, (unsigned)B), dim3(kVcThreads), 0, s, op,
+            B, dinv, r, rc, nsi);
+    return g;
+  }
+  return strips_h(B == 1 ? k_vdown_h<true> : k_vdown_h<false>, nsi, crows, op, B, s, dinv, r, rc);
+}
+static int vup_h(const CoarseOpH& op, int B, const float* dinv, const float* r, const float* ec, float* zout,
+                 cudaStream_t s) {
+  const int nsi = (op.nv / 2 + kVcUpCols - 1) / kVcUpCols;
+  return strips_h(B == 1 ? k_vup_h<true> : k_vup_h<false>, nsi, coarse_strip(nsi, op.nh / 2, B), op, B, s, dinv, r, ec,
+                  zout);
 }
 
 template <class T>
@@ -209,7 +229,7 @@ int launch_vdown(const LevelView<T>& L, int B, const T* lam2, const T* dinv, con
         g = nu == 1 ? vdown_one<FineOpH, float, 1>(L.fh, B, lam2, dinv, r, zpre, rc, ntx, nt, s)
                     : vdown_one<FineOpH, float, 2>(L.fh, B, lam2, dinv, r, zpre, rc, ntx, nt, s);
       else
-        g = nu == 1 ? vdown_h(L.ch, B, dinv, r, zpre, rc, ntx, nt, s)
+        g = nu == 1 ? vdown_h(L.ch, B, dinv, r, rc, s)
                     : vdown_one<CoarseOpH, float, 2>(L.ch, B, lam2, dinv, r, zpre, rc, ntx, nt, s);
       LCMG_LAUNCHED();
       return g;
@@ -247,7 +267,7 @@ int launch_vup(const LevelView<T>& L, int B, const T* lam2, const T* dinv, const
         g = nu == 1 ? vup_one<FineOpH, float, 1>(L.fh, B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s)
                     : vup_one<FineOpH, float, 2>(L.fh, B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
       else
-        g = nu == 1 ? vup_h(L.ch, B, dinv, r, ec, zpre, zout, part, ntx, nt, s)
+        g = nu == 1 ? vup_h(L.ch, B, dinv, r, ec, zout, s)
                     : vup_one<CoarseOpH, float, 2>(L.ch, B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
       LCMG_LAUNCHED();
       return g;
@@ -295,11 +315,12 @@ void launch_vtail(const TailLevelIn* levels, int nlev, const double* kinv, int n
     L.z = in.z;
     const bool coarsest = k == nlev - 1;
     L.o_rows = coarsest ? 0 : take(48 * n);
-    L.o_s = coarsest ? 0 : take(4 * n);
+    L.o_c = coarsest ? 0 : take(4 * n);
     L.o_d = coarsest ? 0 : take(4 * n);
     L.o_r = take(4 * n);
-    L.o_t = coarsest ? 0 : take(4 * n);
-    L.o_res = coarsest ? 0 : take(4 * n);
+    const int np = tail_padded(in.op.nv, in.op.nh);
+    L.o_t = coarsest ? 0 : take(4 * np);
+    L.o_res = coarsest ? 0 : take(4 * np);
     L.o_z = take(4 * n);
   }
   a.kinv = kinv;

