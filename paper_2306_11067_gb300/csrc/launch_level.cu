@@ -71,6 +71,17 @@ void launch_residual(const LevelView<T>& L, int B, const T* lam2, const T* r, co
   LCMG_LAUNCHED();
 }
 
+// multiprocessors of the first device used (all of a system are alike)
+static int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    LCMG_CUDA(cudaGetDevice(&dev));
+    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  }
+  return sms;
+}
+
 // Grid of a tile kernel: every tile once, at most the blocks resident at
 // once on the device and at most kMaxTileBlocks (rows of the partial sums).
 template <class K>
@@ -353,43 +364,35 @@ static int fused_update_grid(int64_t words, int max_blocks) {
 }
 
 // Rows per strip of the row-streaming kernels: at most `most`, and few
-// enough that the strips number about four warps per SM slot of a wave
-// (one warp walks a strip in sequence, so on a small grid long strips leave
-// most of the GPU idle), but at least `least` (the strip's halo rows are
-// computed twice).
-static int strip_rows(int nsi, int len, int most, int least) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    LCMG_CUDA(cudaGetDevice(&dev));
-    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  const int64_t want = (int64_t)sms * 32;  // warps resident at 4 blocks of 8 warps per SM
-  const int64_t per_col = std::max<int64_t>(1, (want + nsi - 1) / nsi);  // strips wanted along the rows
+// enough that the strips make `warps` warps per SM (one warp walks a strip in
+// sequence, so on a small grid long strips leave most of the GPU idle), but at
+// least `least` (the strip's halo rows are computed twice).
+static int strip_rows(int nsi, int B, int len, int warps, int most, int least) {
+  const int64_t want = (int64_t)sm_count() * warps;
+  const int64_t per_col = std::max<int64_t>(1, want / ((int64_t)nsi * B));  // strips wanted along the rows
   const int rows = (int)((len + per_col - 1) / per_col);
   return std::max(least, std::min(most, rows));
 }
+// blocks of 8 warps, or of 2 while the strips are few (so that they spread over the SMs)
+static int strip_threads(int nst, int B) { return (int64_t)nst * B <= 8 * sm_count() ? 64 : kFineThreads; }
 
 int launch_vfine_down(const LevelView<float>& L, int B, const float* lam2, int smoother, double omega,
                       const float* r, float* rc, cudaStream_t s) {
-  const int nt = ((L.nv + kFineTI - 1) / kFineTI) * ((L.nh + kFineTJ - 1) / kFineTJ);
   int g;
-  if (L.h16 && L.nv % 2 == 0 && L.nh % 2 == 0 && (int64_t)L.nv * L.nh * B < (int64_t(1) << 31)) {  // row streaming
-    const int nsi = (L.nv / 2 + kDownCols - 1) / kDownCols;
-    const int crows = strip_rows(nsi, L.nh / 2, kStripCoarse, 2);
+  if (L.h16) {  // row streaming
+    const int nsi = (L.nv / 2 + kFineCols - 1) / kFineCols;
+    const int crows = strip_rows(nsi, B, L.nh / 2, kFineDownWarps, kStripCoarse, 1);
     const int nst = nsi * ((L.nh / 2 + crows - 1) / crows);
     auto k = B == 1 ? k_vfine_down_s<true> : k_vfine_down_s<false>;
-    g = tile_grid(k, kFineThreads, (nst + kFineThreads / 32 - 1) / (kFineThreads / 32));
-    klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fh, B, lam2, smoother, (float)omega, r,
-            rc, nsi, nst, crows);
-  } else if (L.h16) {
-    g = tile_grid(k_vfine_down<FineOpH>, kFineThreads, nt);
-    klaunch(k_vfine_down<FineOpH>, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fh, B, lam2, smoother,
-            (float)omega, r, rc, nt);
+    const int threads = strip_threads(nst, B);
+    g = std::min((nst + threads / 32 - 1) / (threads / 32), kMaxTileBlocks);
+    klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(threads), 0, s, L.fh, B, lam2, smoother, (float)omega, r, rc, nsi,
+            nst, crows);
   } else {
-    g = tile_grid(k_vfine_down<FineOp<float>>, kFineThreads, nt);
-    klaunch(k_vfine_down<FineOp<float>>, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fine_op(), B,
-            lam2, smoother, (float)omega, r, rc, nt);
+    const int nt = ((L.nv + kFineTI - 1) / kFineTI) * ((L.nh + kFineTJ - 1) / kFineTJ);
+    g = tile_grid(k_vfine_down, kFineThreads, nt);
+    klaunch(k_vfine_down, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fine_op(), B, lam2, smoother,
+            (float)omega, r, rc, nt);
   }
   LCMG_LAUNCHED();
   return g;
@@ -397,24 +400,21 @@ int launch_vfine_down(const LevelView<float>& L, int B, const float* lam2, int s
 
 int launch_vfine_up(const LevelView<float>& L, int B, const float* lam2, int smoother, double omega,
                     const float* r, const float* ec, float* zout, double* part, cudaStream_t s) {
-  const int nt = ((L.nv + kFineTI - 1) / kFineTI) * ((L.nh + kFineTJ - 1) / kFineTJ);
   int g;
-  if (L.h16 && L.nv % 2 == 0 && L.nh % 2 == 0 && (int64_t)L.nv * L.nh * B < (int64_t(1) << 31)) {  // row streaming
-    const int nsi = (L.nv + kUpCols - 1) / kUpCols;
-    const int rows = strip_rows(nsi, L.nh, kStripRows, 4);
+  if (L.h16) {  // row streaming
+    const int nsi = (L.nv / 2 + kFineCols - 1) / kFineCols;
+    const int rows = strip_rows(nsi, B, L.nh, kFineUpWarps, kStripRows, 2);
     const int nst = nsi * ((L.nh + rows - 1) / rows);
     auto k = B == 1 ? k_vfine_up_s<true> : k_vfine_up_s<false>;
-    g = tile_grid(k, kFineThreads, (nst + kFineThreads / 32 - 1) / (kFineThreads / 32));
-    klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fh, B, lam2, smoother, (float)omega, r,
-            ec, zout, nsi, nst, rows, part);
-  } else if (L.h16) {
-    g = tile_grid(k_vfine_up<FineOpH>, kFineThreads, nt);
-    klaunch(k_vfine_up<FineOpH>, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fh, B, lam2, smoother,
-            (float)omega, r, ec, zout, nt, part);
+    const int threads = strip_threads(nst, B);
+    g = std::min((nst + threads / 32 - 1) / (threads / 32), kMaxTileBlocks);
+    klaunch(k, dim3((unsigned)g, (unsigned)B), dim3(threads), 0, s, L.fh, B, lam2, smoother, (float)omega, r, ec, zout,
+            nsi, nst, rows, part);
   } else {
-    g = tile_grid(k_vfine_up<FineOp<float>>, kFineThreads, nt);
-    klaunch(k_vfine_up<FineOp<float>>, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fine_op(), B,
-            lam2, smoother, (float)omega, r, ec, zout, nt, part);
+    const int nt = ((L.nv + kFineTI - 1) / kFineTI) * ((L.nh + kFineTJ - 1) / kFineTJ);
+    g = tile_grid(k_vfine_up, kFineThreads, nt);
+    klaunch(k_vfine_up, dim3((unsigned)g, (unsigned)B), dim3(kFineThreads), 0, s, L.fine_op(), B, lam2, smoother,
+            (float)omega, r, ec, zout, nt, part);
   }
   LCMG_LAUNCHED();
   return g;

@@ -13,13 +13,15 @@
 //   k_vfine_down: z1 = D^{-1} r, res = r - K z1, r_c = P^T res
 //   k_vfine_up:   z0 = z1 + P e_c, z = z0 + D^{-1} (r - K z0), partials r.z
 //
-// A block owns a 64 x 32 tile of fine points (a 32 x 16 tile of coarse
-// points) and keeps the windows its stencils need in shared memory
+// FP32 weights: a block owns a 64 x 32 tile of fine points (a 32 x 16 tile
+// of coarse points) and keeps the windows its stencils need in shared memory
 // (halo 2 for the down kernel, 1 for the up kernel); blocks stride over the
-// tiles.  The sums per point are those of the generic tile kernels.
+// tiles.  The sums per point are those of the generic tile kernels.  FP16
+// weights: the row-streaming kernels at the end.
 #pragma once
 #include "compact.cuh"
 #include "kernels.cuh"
+#include "vcoarse.cuh"
 
 namespace lcmg {
 
@@ -27,27 +29,18 @@ constexpr int kFineTI = 64;  // fine points per tile along i (contiguous)
 constexpr int kFineTJ = 32;  // ... along j
 constexpr int kFineThreads = 256;
 
-// the stored fine-level weights of either operator form
-__device__ __forceinline__ float fw_s(const FineOp<float>& op, int64_t p) { return op.ws[p]; }
-__device__ __forceinline__ float fw_e(const FineOp<float>& op, int64_t p) { return op.we[p]; }
-__device__ __forceinline__ float fw_g(const FineOp<float>& op, int64_t p) { return op.ga[p]; }
-__device__ __forceinline__ float fw_s(const FineOpH& op, int64_t p) { return op.ws_(p); }
-__device__ __forceinline__ float fw_e(const FineOpH& op, int64_t p) { return op.we_(p); }
-__device__ __forceinline__ float fw_g(const FineOpH& op, int64_t p) { return op.ga_(p); }
-
 // the four edge weights around point (i, j) (zero across the boundary) and
 // diag(A^T A) there
 struct FineW {
   float s, n, e, w, g;
 };
-template <class Op>
-__device__ __forceinline__ FineW fine_w(const Op& op, int64_t p, int i, int j) {
+__device__ __forceinline__ FineW fine_w(const FineOp<float>& op, int64_t p, int i, int j) {
   FineW f;
-  f.s = i + 1 < op.nv ? fw_s(op, p) : 0.f;
-  f.n = i > 0 ? fw_s(op, p - 1) : 0.f;
-  f.e = j + 1 < op.nh ? fw_e(op, p) : 0.f;
-  f.w = j > 0 ? fw_e(op, p - op.nv) : 0.f;
-  f.g = fw_g(op, p);
+  f.s = i + 1 < op.nv ? op.ws[p] : 0.f;
+  f.n = i > 0 ? op.ws[p - 1] : 0.f;
+  f.e = j + 1 < op.nh ? op.we[p] : 0.f;
+  f.w = j > 0 ? op.we[p - op.nv] : 0.f;
+  f.g = op.ga[p];
   return f;
 }
 
@@ -64,9 +57,8 @@ __device__ __forceinline__ float fine_kz(const FineW& f, float l2, const float* 
   return l2 * acc + f.g * zp;
 }
 
-template <class Op>
 __global__ void __launch_bounds__(kFineThreads)
-    k_vfine_down(Op op, int B, const float* __restrict__ lam2, int smoother, float omega,
+    k_vfine_down(FineOp<float> op, int B, const float* __restrict__ lam2, int smoother, float omega,
                  const float* __restrict__ r, float* __restrict__ rc, int ntiles) {
   constexpr int ZI = kFineTI + 4, ZJ = kFineTJ + 4;  // z1 window, halo 2
   constexpr int RI = kFineTI + 2, RJ = kFineTJ + 2;  // residual window, halo 1
@@ -126,9 +118,8 @@ __global__ void __launch_bounds__(kFineThreads)
   }
 }
 
-template <class Op>
 __global__ void __launch_bounds__(kFineThreads)
-    k_vfine_up(Op op, int B, const float* __restrict__ lam2, int smoother, float omega,
+    k_vfine_up(FineOp<float> op, int B, const float* __restrict__ lam2, int smoother, float omega,
                const float* __restrict__ r, const float* __restrict__ ec, float* __restrict__ zout, int ntiles,
                double* __restrict__ part) {
   constexpr int WI = kFineTI + 2, WJ = kFineTJ + 2;          // z0 window, halo 1
@@ -209,245 +200,254 @@ __global__ void __launch_bounds__(kFineThreads)
 
 
 // ---------------------------------------------------------------------------
-// Row-streaming forms of the two FP16 kernels (the default).  A warp owns
-// 32 consecutive points along i (one per lane) and walks down a strip of
-// rows j: the neighbours along j of the point a lane is at are values it
-// computed one row earlier or one row ahead (kept in registers), those
-// along i are the neighbouring lanes' values (warp shuffles).  The two edge
-// lanes of a warp compute only what their neighbours need (the halo), so a
-// warp produces 30 points of z (k_vfine_up_s) or 14 coarse points of r_c
-// (k_vfine_down_s) per row; a strip is at most kStripRows rows (kStripCoarse
-// coarse rows), fewer on small grids, so that the strips fill the GPU.  No
-// shared memory, no barrier; a row's loads
-// are issued one row ahead of their use, from addresses clamped into the
-// arrays, and every per-point step is branch-free (selects), so that a
-// lane's work per row is its arithmetic and little else.
+// Row-streaming forms of the two kernels for the FP16 weights.  A warp owns
+// 64 consecutive points along i, two per lane (a coarse column's own pair),
+// and walks down a strip of rows j: the neighbours along j are values the
+// lane computed one row earlier or one row ahead (kept in registers), those
+// along i are the lane's other point or the neighbouring lanes' (shuffles).
+// The edge lanes compute only what their neighbours need (the halo), so a
+// warp produces 60 points of z (k_vfine_up_s) or 30 coarse points of r_c
+// (k_vfine_down_s) per row.  No shared memory, no barrier; a row's loads are
+// issued one row ahead of their use, from addresses clamped into the arrays.
+// The weights are zero on the last row and column and outside the grid, so
+// no step tests for the edge.
 //
-// Each point's formulas are those of k_vfine_up / k_vfine_down, with two
+// What bounds them: HBM at 2048^2 points (46 and 63 MB per launch), below
+// 512^2 the latency of a row's loads; with one point per lane it was the
+// instructions (165 per warp and row of 30 points).  Measured on GB300 against
+// that form, down / up: 2048^2 27.4 / 34.9 -> 18.5 / 24.1 us, 512^2 in four
+// columns 12.6 / 13.4 -> 8.0 / 10.4 us, 256^2 3.9 / 3.9 -> 3.5 / 3.8 us.  With as
+// many strips as 16 / 8, 24 / 16 and 32 / 32 warps per SM: 23.2 / 25.4, 18.3 /
+// 24.2, 25.7 / 26.2 us at 2048^2.
+//
+// Each point's formulas are those of k_vfine_up / k_vfine_down, with three
 // changes of rounding: D^{-1} = 1 / (2 lam^2 sum w + g) (or omega / (lam^2
 // sum w + g)) is taken with the fast division (__fdividef, within 2 ulp),
 // the same value in both kernels, so the cycle stays one fixed symmetric
-// operator; and r_c = P^T res is summed per fine row along i first, then
-// along j.  32-bit indices: the launcher takes this path while
-// n_v n_h B < 2^31.
+// operator; r_c = P^T res is summed per fine row along i first, then along
+// j; and P e_c along j first.
 // ---------------------------------------------------------------------------
 constexpr int kStripRows = 32;    // most fine rows of z per k_vfine_up_s strip
 constexpr int kStripCoarse = 16;  // most coarse rows of r_c per k_vfine_down_s strip
-constexpr int kUpCols = 30;       // z columns per warp
-constexpr int kDownCols = 14;     // r_c columns per warp
+constexpr int kFineCols = 30;     // coarse columns (pairs) per warp
+constexpr int kFineDownWarps = 24;  // warps per SM the strips aim at (those resident)
+constexpr int kFineUpWarps = 16;
 
-// the raw data of the lane's point p = i + j n_v of one row: FP16 w_s(p),
-// w_s(p - 1), w_e(p), diag(A^T A)(p), r(p) and, for the up kernel, the four
-// coarse corrections of P e_c (element stride S of the interleaved vectors)
-struct RawRow {
-  __half s, n, e, g;
-  float r;
-  float c[4];
+// the stored data of a lane's pair in one row: FP16 w_s, w_e, diag(A^T A),
+// w_s of the point before the pair (lane 0 alone reads it, the others have
+// it from their neighbour), r
+struct FineRaw {
+  __half2 s, e, g;
+  __half n;
+  Pair r;
 };
-template <bool kCoarse>
-__device__ __forceinline__ RawRow fine_load(const __half* __restrict__ ws, const __half* __restrict__ we,
-                                            const __half* __restrict__ ga, const float* __restrict__ r,
-                                            const float* __restrict__ ec, int S, int col, bool in, int p, int ea,
-                                            int eb, int Iac, int Ibc) {
-  RawRow q;
-  const int pc = in ? p : 0;
-  q.s = ws[pc];
-  q.n = ws[pc > 0 ? pc - 1 : 0];
-  q.e = we[pc];
-  q.g = ga[pc];
-  q.r = r[pc * S + col];
-  if (kCoarse) {
-    q.c[0] = ec[(ea + Iac) * S + col];
-    q.c[1] = ec[(ea + Ibc) * S + col];
-    q.c[2] = ec[(eb + Iac) * S + col];
-    q.c[3] = ec[(eb + Ibc) * S + col];
-  }
-  return q;
-}
-
-// the point data a lane carries from one row to the next
-struct FineRow {
-  float z;     // z1 = D^{-1} r (down) or z0 = z1 + P e_c (up)
-  float r, d;  // r and D^{-1}
-  float s, n, e, w, g;
+// what a lane carries from one row to the next
+struct FinePair {
+  Pair z;       // z1 = D^{-1} r (down) or z0 = z1 + P e_c (up)
+  Pair r, d;    // r and D^{-1}
+  float2 s, e;  // w_s, w_e (in stored units)
+  float n;      // w_s of the point before the pair
+  float2 w;     // w_e of the row before
+  float2 g;     // diag(A^T A)
 };
-
-// weights, D^{-1} and z1 of the lane's point (all zero outside the grid);
-// w_prev = e of (i, j - 1)
-__device__ __forceinline__ FineRow fine_row(const RawRow& q, float sw, float sg, float l2, int smoother, float omega,
-                                            bool in, bool has_s, bool has_n, bool has_e, float w_prev) {
-  FineRow f;
-  f.s = (in && has_s) ? __half2float(q.s) * sw : 0.f;
-  f.n = (in && has_n) ? __half2float(q.n) * sw : 0.f;
-  f.e = (in && has_e) ? __half2float(q.e) * sw : 0.f;
-  f.w = w_prev;
-  f.g = in ? __half2float(q.g) * sg : 0.f;
-  f.r = in ? q.r : 0.f;
-  const float sum = f.s + f.n + f.e + f.w;
-  const float dv = smoother == 0 ? __fdividef(1.0f, 2.0f * l2 * sum + f.g) : __fdividef(omega, l2 * sum + f.g);
-  f.d = in ? dv : 0.f;
-  f.z = f.d * f.r;
-  return f;
-}
-
-// (K z)_p from the lane's row record and its neighbours' z
-__device__ __forceinline__ float fine_row_kz(const FineRow& f, float l2, float zs, float zn, float ze, float zw) {
-  const float zp = f.z;
-  const float acc = f.s * (zp - zs) + f.n * (zp - zn) + f.e * (zp - ze) + f.w * (zp - zw);
-  return l2 * acc + f.g * zp;
-}
-
-// pw1 of the two coarse neighbours of fine index a on a line of n = 2 nc
-// points: the nearer one (3/4, or 1 at the ends of the line) and the other
-// one (1/4, or 0 at the ends, where it falls outside)
-__device__ __forceinline__ void pw1_pair(int a, int n, float& wnear, float& wfar) {
-  const bool edge = a == 0 || a == n - 1;
-  wnear = edge ? 1.f : 0.75f;
-  wfar = edge ? 0.f : 0.25f;
-}
 
 template <bool kUnit>
-__global__ void __launch_bounds__(kFineThreads)
+struct FineStream {
+  FineOpH op;
+  const float* __restrict__ r;
+  int B, col, smoother;
+  float l2s, sg, omega;  // lam^2 in the units of the stored weights
+  int lane, i;           // the lane's pair (i, i + 1), clamped into the row
+  bool in_i;
+
+  __device__ __forceinline__ FineRaw load(int j) const {
+    FineRaw q;
+    const int64_t e = (int64_t)i + (int64_t)min(max(j, 0), op.nh - 1) * op.nv;
+    q.s = *reinterpret_cast<const __half2*>(op.ws + e);
+    q.e = *reinterpret_cast<const __half2*>(op.we + e);
+    q.g = *reinterpret_cast<const __half2*>(op.ga + e);
+    q.n = __half(0);
+    if (lane == 0 && i > 0) q.n = op.ws[e - 1];
+    q.r = ld_pair<kUnit>(r, e, B, col);
+    return q;
+  }
+  // w_e of row j (zero outside the grid)
+  __device__ __forceinline__ float2 edge(int j) const {
+    if (!in_i || j < 0 || j >= op.nh) return make_float2(0.f, 0.f);
+    return __half22float2(*reinterpret_cast<const __half2*>(op.we + (int64_t)i + (int64_t)j * op.nv));
+  }
+  // weights, D^{-1} and z1 of row j (all zero outside the grid); w = edge(j - 1)
+  __device__ __forceinline__ FinePair row(const FineRaw& q, int j, const float2 w) const {
+    FinePair f;
+    const bool in = in_i && j >= 0 && j < op.nh;
+    const float2 zero = make_float2(0.f, 0.f);
+    f.s = in ? __half22float2(q.s) : zero;
+    f.e = in ? __half22float2(q.e) : zero;
+    f.g = in ? __half22float2(q.g) : zero;
+    f.g.x *= sg;
+    f.g.y *= sg;
+    f.w = w;
+    f.n = __shfl_up_sync(0xffffffffu, f.s.y, 1);
+    if (lane == 0) f.n = in ? __half2float(q.n) : 0.f;
+    f.r.a = in ? q.r.a : 0.f;
+    f.r.b = in ? q.r.b : 0.f;
+    const float sa = f.s.x + f.n + f.e.x + f.w.x, sb = f.s.y + f.s.x + f.e.y + f.w.y;
+    if (smoother == 0) {
+      f.d.a = __fdividef(1.0f, 2.0f * l2s * sa + f.g.x);
+      f.d.b = __fdividef(1.0f, 2.0f * l2s * sb + f.g.y);
+    } else {
+      f.d.a = __fdividef(omega, l2s * sa + f.g.x);
+      f.d.b = __fdividef(omega, l2s * sb + f.g.y);
+    }
+    if (!in) f.d.a = f.d.b = 0.f;
+    f.z.a = f.d.a * f.r.a;
+    f.z.b = f.d.b * f.r.b;
+    return f;
+  }
+  // (K z) at the pair of row f, zm and zp the pairs of the rows before and after
+  __device__ __forceinline__ Pair kz(const FinePair& f, const Pair& zm, const Pair& zp) const {
+    const float zl = __shfl_up_sync(0xffffffffu, f.z.b, 1), zr = __shfl_down_sync(0xffffffffu, f.z.a, 1);
+    const float a = f.s.x * (f.z.a - f.z.b) + f.n * (f.z.a - zl) + f.e.x * (f.z.a - zp.a) + f.w.x * (f.z.a - zm.a);
+    const float b = f.s.y * (f.z.b - zr) + f.s.x * (f.z.b - f.z.a) + f.e.y * (f.z.b - zp.b) + f.w.y * (f.z.b - zm.b);
+    return {l2s * a + f.g.x * f.z.a, l2s * b + f.g.y * f.z.b};
+  }
+};
+
+template <bool kUnit>
+__global__ void __launch_bounds__(kFineThreads, 2)
     k_vfine_up_s(FineOpH op, int B, const float* __restrict__ lam2, int smoother, float omega,
                  const float* __restrict__ r, const float* __restrict__ ec, float* __restrict__ zout, int nsi,
                  int nstrips, int rows, double* __restrict__ part) {
   __shared__ double sred[kFineThreads / 32];
-  const unsigned FULL = 0xffffffffu;
-  const int S = kUnit ? 1 : B;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int col = blockIdx.y;
   const int nv = op.nv, nh = op.nh, nvc = nv / 2, nhc = nh / 2;
-  const __half* __restrict__ ws = op.ws;
-  const __half* __restrict__ we = op.we;
-  const __half* __restrict__ ga = op.ga;
-  const float sw = op.sw, sg = op.sg;
-  const float l2 = lam2[col];
   Dot2 dot;
-  for (int st = blockIdx.x * (kFineThreads / 32) + warp; st < nstrips; st += gridDim.x * (kFineThreads / 32)) {
-    const int i = (st % nsi) * kUpCols - 1 + lane;
-    const int j0 = (st / nsi) * rows, j1 = min(j0 + rows, nh);
-    const bool in_i = i >= 0 && i < nv, has_s = i + 1 < nv, has_n = i > 0;
-    const bool out = lane >= 1 && lane <= kUpCols && i < nv;
-    // interpolation along i (fixed for the lane): coarse columns Ia, Ib
-    const int Ia = i >> 1;
-    float waA, waB;
-    pw1_pair(i, nv, waA, waB);
-    const int Iac = min(max(Ia, 0), nvc - 1);
-    const int Ibc = min(max((i & 1) ? Ia + 1 : Ia - 1, 0), nvc - 1);
-    auto load = [&](int j, int q) {
-      const int Ja = min(max(j >> 1, 0), nhc - 1);
-      const int Jb = min(max((j & 1) ? Ja + 1 : Ja - 1, 0), nhc - 1);
-      return fine_load<true>(ws, we, ga, r, ec, S, col, in_i && j >= 0 && j < nh, q, Ja * nvc, Jb * nvc, Iac, Ibc);
+  for (int st = blockIdx.x * (blockDim.x >> 5) + warp; st < nstrips; st += gridDim.x * (blockDim.x >> 5)) {
+    const int I = st % nsi * kFineCols - 1 + lane;
+    const int j0 = st / nsi * rows, j1 = min(j0 + rows, nh);
+    const bool in_i = I >= 0 && I < nvc;
+    const int Ic = in_i ? I : 0;
+    const FineStream<kUnit> F{op, r, B, col, smoother, lam2[col] * op.sw, op.sg, omega, lane, 2 * Ic, in_i};
+    const bool out = in_i && lane >= 1 && lane <= kFineCols;
+    // interpolation along i (fixed for the lane): columns I, I - 1 and I + 1
+    const int Il = max(Ic - 1, 0), Ir = min(Ic + 1, nvc - 1);
+    float na, fa, nb, fb;
+    pw1_near_far(2 * Ic, nv, na, fa);
+    pw1_near_far(2 * Ic + 1, nv, nb, fb);
+    struct Corr {
+      float e[2][3];  // e_c of the nearer and the other coarse row at I - 1, I, I + 1
+    };
+    auto load_c = [&](int j) {
+      Corr q;
+      const int jc = min(max(j, 0), nh - 1);
+      const int Ja = jc >> 1, Jb = min(max((jc & 1) ? Ja + 1 : Ja - 1, 0), nhc - 1);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int64_t e = (int64_t)(u ? Jb : Ja) * nvc;
+        const int S = kUnit ? 1 : B, co = kUnit ? 0 : col;
+        q.e[u][0] = ec[(e + Il) * S + co];
+        q.e[u][1] = ec[(e + Ic) * S + co];
+        q.e[u][2] = ec[(e + Ir) * S + co];
+      }
+      return q;
     };
     // z0 = D^{-1} r + P e_c at row j (zero outside the grid)
-    auto row = [&](const RawRow& q, int j, float w_prev) {
-      const bool in = in_i && j >= 0 && j < nh;
-      FineRow f = fine_row(q, sw, sg, l2, smoother, omega, in, has_s, has_n, j + 1 < nh, w_prev);
-      float wbA, wbB;
-      pw1_pair(j, nh, wbA, wbB);
-      float acc = 0.f;  // the terms in the order of k_vfine_up (a zero weight adds nothing)
-      acc += wbA * waA * q.c[0];
-      acc += wbA * waB * q.c[1];
-      acc += wbB * waA * q.c[2];
-      acc += wbB * waB * q.c[3];
-      f.z += in ? acc : 0.f;
+    auto row = [&](const FineRaw& q, const Corr& c, int j, const float2 w) {
+      FinePair f = F.row(q, j, w);
+      float wn, wf;
+      pw1_near_far(j, nh, wn, wf);
+      if (!in_i || j < 0 || j >= nh) wn = wf = 0.f;
+      const float c0 = wn * c.e[0][0] + wf * c.e[1][0];
+      const float c1 = wn * c.e[0][1] + wf * c.e[1][1];
+      const float c2 = wn * c.e[0][2] + wf * c.e[1][2];
+      f.z.a += na * c1 + fa * c0;
+      f.z.b += nb * c1 + fb * c2;
       return f;
     };
-    int p = i + (j0 - 1) * nv;  // the lane's point in row j0 - 1
-    float we_prev = 0.f;        // e of the row above, the w of the next row
-    if (j0 - 2 >= 0 && in_i && j0 - 1 < nh) we_prev = __half2float(we[p - nv]) * sw;
-    RawRow qn = load(j0 + 1, p + 2 * nv);  // in flight while rows j0 - 1 and j0 are finished
-    FineRow fm = row(load(j0 - 1, p), j0 - 1, we_prev);
-    p += nv;
-    FineRow fc = row(load(j0, p), j0, fm.e);
+    // every first load is issued before the first shuffle
+    const FineRaw qa = F.load(j0 - 1), qb = F.load(j0);
+    const Corr ca = load_c(j0 - 1), cb = load_c(j0);
+    const float2 ea = F.edge(j0 - 2);
+    FineRaw qn = F.load(j0 + 1);
+    Corr cn = load_c(j0 + 1);
+    FinePair fm = row(qa, ca, j0 - 1, ea);
+    FinePair fc = row(qb, cb, j0, fm.e);
+#pragma unroll 3
     for (int j = j0; j < j1; ++j) {
-      const RawRow qj = qn;
-      qn = load(j + 2, p + 2 * nv);  // the loads of the row after next
-      const FineRow fp = row(qj, j + 1, fc.e);
-      const float zs = __shfl_down_sync(FULL, fc.z, 1);
-      const float zn = __shfl_up_sync(FULL, fc.z, 1);
-      const float zn1 = fc.z + fc.d * (fc.r - fine_row_kz(fc, l2, zs, zn, fp.z, fm.z));
-      if (out) zout[p * S + col] = zn1;
-      dot.add(out ? fc.r : 0.f, out ? zn1 : 0.f);
+      const FineRaw qj = qn;
+      const Corr cj = cn;
+      qn = F.load(j + 2);  // the loads of the row after next
+      cn = load_c(j + 2);
+      const FinePair fp = row(qj, cj, j + 1, fc.e);
+      const Pair kz = F.kz(fc, fm.z, fp.z);
+      const float za = fc.z.a + fc.d.a * (fc.r.a - kz.a), zb = fc.z.b + fc.d.b * (fc.r.b - kz.b);
+      if (out) {
+        const int64_t e = (int64_t)(2 * I) + (int64_t)j * nv;
+        if (kUnit) {
+          *reinterpret_cast<float2*>(zout + e) = make_float2(za, zb);
+        } else {
+          zout[e * B + col] = za;
+          zout[(e + 1) * B + col] = zb;
+        }
+        dot.add(fc.r.a, za);
+        dot.add(fc.r.b, zb);
+      }
       fm = fc;
       fc = fp;
-      p += nv;
     }
   }
   if (part) {
-    double dacc = dot.value();
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) dacc += __shfl_xor_sync(FULL, dacc, off);
+    const double dacc = dot.warp_sum();
     if (lane == 0) sred[warp] = dacc;
     __syncthreads();
     if (threadIdx.x == 0) {
       double sum = 0.0;
-      for (int k = 0; k < kFineThreads / 32; ++k) sum += sred[k];
+      for (int k = 0; k < (int)blockDim.x >> 5; ++k) sum += sred[k];
       part[(int64_t)blockIdx.x * B + col] = sum;
     }
   }
 }
 
 template <bool kUnit>
-__global__ void __launch_bounds__(kFineThreads)
+__global__ void __launch_bounds__(kFineThreads, 3)
     k_vfine_down_s(FineOpH op, int B, const float* __restrict__ lam2, int smoother, float omega,
                    const float* __restrict__ r, float* __restrict__ rc, int nsi, int nstrips, int crows) {
   const unsigned FULL = 0xffffffffu;
-  const int S = kUnit ? 1 : B;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int col = blockIdx.y;
-  const int nv = op.nv, nh = op.nh, nvc = nv / 2, nhc = nh / 2;
-  const __half* __restrict__ ws = op.ws;
-  const __half* __restrict__ we = op.we;
-  const __half* __restrict__ ga = op.ga;
-  const float sw = op.sw, sg = op.sg;
-  const float l2 = lam2[col];
-  for (int st = blockIdx.x * (kFineThreads / 32) + warp; st < nstrips; st += gridDim.x * (kFineThreads / 32)) {
-    const int I0 = (st % nsi) * kDownCols, J0 = (st / nsi) * crows;
-    const int i = 2 * I0 - 2 + lane;  // z1 at every lane, res at lanes 1..30
-    const bool in_i = i >= 0 && i < nv, has_s = i + 1 < nv, has_n = i > 0;
-    // restriction along i: coarse column I = I0 + lane (lanes < 14) from the
-    // residual at fine columns 2I - 1 .. 2I + 2 (lanes 2 lane + 1 .. 2 lane + 4)
-    const int I = I0 + lane;
-    const bool out = lane < kDownCols && I < nvc;
-    float wa[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int a2 = 2 * I - 1 + m;
-      wa[m] = (a2 >= 0 && a2 < nv && I < nvc) ? pw1<float>(a2, I, nvc) : 0.f;
-    }
-    const int jb0 = 2 * J0 - 1, jb1 = min(2 * (J0 + crows), nh);  // residual rows [jb0, jb1]
-    int p = i + (jb0 - 1) * nv;  // the lane's point in row jb0 - 1
-    float we_prev = 0.f;
-    if (jb0 - 2 >= 0 && in_i && jb0 - 1 < nh) we_prev = __half2float(we[p - nv]) * sw;
-    auto load = [&](int j, int q) {
-      return fine_load<false>(ws, we, ga, r, nullptr, S, col, in_i && j >= 0 && j < nh, q, 0, 0, 0, 0);
-    };
-    auto row = [&](const RawRow& q, int j, float w_prev) {
-      return fine_row(q, sw, sg, l2, smoother, omega, in_i && j >= 0 && j < nh, has_s, has_n, j + 1 < nh, w_prev);
-    };
-    RawRow qn = load(jb0 + 1, p + 2 * nv);  // in flight while rows jb0 - 1 and jb0 are finished
-    FineRow fm = row(load(jb0 - 1, p), jb0 - 1, we_prev);
-    p += nv;
-    FineRow fc = row(load(jb0, p), jb0, fm.e);
+  const int nh = op.nh, nvc = op.nv / 2, nhc = nh / 2;
+  for (int st = blockIdx.x * (blockDim.x >> 5) + warp; st < nstrips; st += gridDim.x * (blockDim.x >> 5)) {
+    const int I = st % nsi * kFineCols - 1 + lane;  // z1 at every lane, r_c at lanes 1..30
+    const int J0 = st / nsi * crows, J1 = min(J0 + crows, nhc);
+    const bool in_i = I >= 0 && I < nvc;
+    const FineStream<kUnit> F{op, r, B, col, smoother, lam2[col] * op.sw, op.sg, omega, lane, in_i ? 2 * I : 0, in_i};
+    const bool out = in_i && lane >= 1 && lane <= kFineCols;
+    // restriction along i from the residuals at 2I - 1 .. 2I + 2
+    const float w1 = I == 0 ? 1.f : 0.75f, w2 = I == nvc - 1 ? 1.f : 0.75f;
+    const int b0 = 2 * J0 - 1, b1 = 2 * J1;  // residual rows
+    // every first load is issued before the first shuffle
+    const FineRaw q0 = F.load(b0 - 1), q1 = F.load(b0);
+    const float2 ea = F.edge(b0 - 2);
+    FineRaw qn = F.load(b0 + 1);
+    FinePair fm = F.row(q0, b0 - 1, ea);
+    FinePair fc = F.row(q1, b0, fm.e);
     float prev = 0.f, cur = 0.f;  // r_c of coarse rows (b - 1) / 2 and (b + 1) / 2 being summed
-    for (int b = jb0; b <= jb1; ++b) {
-      const RawRow qb = qn;
-      qn = load(b + 2, p + 2 * nv);  // the loads of the row after next
-      const FineRow fp = row(qb, b + 1, fc.e);
-      const float zs = __shfl_down_sync(FULL, fc.z, 1);
-      const float zn = __shfl_up_sync(FULL, fc.z, 1);
-      // res = r - K z1, zero outside the grid (so that it adds nothing below)
-      const bool in = in_i && b >= 0 && b < nh;
-      const float res = in ? fc.r - fine_row_kz(fc, l2, zs, zn, fp.z, fm.z) : 0.f;
-      float ti = 0.f;  // sum over a of pw1(a, I) res(a, b)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) ti += wa[m] * __shfl_sync(FULL, res, (2 * lane + 1 + m) & 31);
-      const float wb = (b == 0 || b == nh - 1) ? 1.f : 0.75f;  // pw1(b, b / 2)
+#pragma unroll 3
+    for (int b = b0; b <= b1; ++b) {
+      const FineRaw qb = qn;
+      qn = F.load(b + 2);  // the loads of the row after next
+      const FinePair fp = F.row(qb, b + 1, fc.e);
+      const Pair kz = F.kz(fc, fm.z, fp.z);
+      // res = r - K z1 (zero outside the grid: every term is)
+      const float ra = fc.r.a - kz.a, rb = fc.r.b - kz.b;
+      const float left = __shfl_up_sync(FULL, rb, 1), right = __shfl_down_sync(FULL, ra, 1);
+      const float ti = 0.25f * left + w1 * ra + w2 * rb + 0.25f * right;  // sum over a of pw1(a, I) res(a, b)
+      const float wb = (b == 0 || b == nh - 1) ? 1.f : 0.75f;             // pw1(b, b / 2)
       const int m = b >> 1;
       if ((b & 1) == 0) {  // b = 2m: the last term of coarse row m - 1, the second of row m
         prev += 0.25f * ti;
-        if (out && m - 1 >= J0 && m - 1 < nhc) rc[(I + (m - 1) * nvc) * S + col] = prev;
+        if (out && m - 1 >= J0) rc[((int64_t)I + (int64_t)(m - 1) * nvc) * B + col] = prev;
         prev = cur + wb * ti;
         cur = 0.f;
       } else {  // b = 2m + 1: the third term of row m, the first of row m + 1
@@ -456,7 +456,6 @@ __global__ void __launch_bounds__(kFineThreads)
       }
       fm = fc;
       fc = fp;
-      p += nv;
     }
   }
 }
