@@ -1005,14 +1005,20 @@ __global__ void __launch_bounds__(kBlock)
 // per SM, since every block repeats the FP64 sums (the FP64 pipe runs at a
 // small fraction of the FP32 one), which four warps share.  Measured on
 // GB300 at 2048^2 in FP32, against scalar loads in a grid of four blocks of
-// 256 threads per SM whose first warp summed alone: 33.7 -> 14.6 us (the 101
-// MB take 14.8 from HBM) and 21.8 -> 10.7 us (50 MB, 7.4).
+// 256 threads per SM whose first warp summed alone: 33.7 -> 14.0 us (the 101
+// MB take 14.8 from HBM) and 21.8 -> 9.7 us (50 MB, 7.4).
+//
+// At small n an FP64 warp instruction holds an SM for 19 cycles, so there are
+// few of them: blocks of 256 threads, the block's r.r combined through shared
+// memory by one warp (21 instead of 84), and the column state read before the
+// sums rather than in the decision that follows them.  64 x 64 in FP64, against
+// blocks of 512 and a shuffle tree per warp: 5.1 -> 4.3 and 4.9 -> 4.0 us.
 constexpr int kUpdThreads = 512;
 constexpr int kSumWarps = 4;  // warps that share one sum of partials
 
-// This warp's share (warp wq of kSumWarps) of the sum of nb partials, in a
-// fixed order, the same in every block; valid in every lane.
-__device__ __forceinline__ double part_share(const double* __restrict__ part, int nb, int wq) {
+// This warp's share (warp wq of kSumWarps) of the sum of nb partials of one of
+// B columns, in a fixed order, the same in every block; valid in every lane.
+__device__ __forceinline__ double part_share(const double* __restrict__ part, int nb, int wq, int B = 1, int col = 0) {
   constexpr int U = 8;  // loads in flight
   const int lane = threadIdx.x & 31;
   double s = 0.0;
@@ -1021,7 +1027,7 @@ __device__ __forceinline__ double part_share(const double* __restrict__ part, in
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int b = base + (u * kSumWarps + wq) * 32 + lane;
-      v[u] = b < nb ? part[b] : 0.0;
+      v[u] = b < nb ? part[(int64_t)b * B + col] : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -1064,10 +1070,10 @@ __global__ void __launch_bounds__(kUpdThreads)
   __shared__ double s_al;
   __shared__ int s_ok;
   __shared__ double s_pq[kSumWarps];
-  __shared__ double sm[kUpdThreads / 32];
+  __shared__ double sm[kUpdThreads];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t nv = n / P::W, stride = (int64_t)gridDim.x * kUpdThreads;
-  int64_t i = (int64_t)blockIdx.x * kUpdThreads + threadIdx.x;
+  const int64_t nv = n / P::W, stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   P xv[2], rv[2], pv[2], qv[2];
   auto load = [&](int64_t at) {
 #pragma unroll
@@ -1080,7 +1086,7 @@ __global__ void __launch_bounds__(kUpdThreads)
       }
   };
   load(i);
-  const int act = st.active[0];
+  const int act = st.active[0], its = st.iters[0];
   const double rzc = st.rz2[0];
   if (warp < kSumWarps) {
     const double s = part_share(pq_part, nb_pq, warp);
@@ -1100,7 +1106,7 @@ __global__ void __launch_bounds__(kUpdThreads)
       st.counters[2] = 0;
       st.alpha[0] = al;
       if (act) {
-        st.iters[0] += 1;
+        st.iters[0] = its + 1;
         if (!fin) {
           st.status[0] = ST_NONFINITE;
           st.active[0] = 0;
@@ -1138,15 +1144,12 @@ __global__ void __launch_bounds__(kUpdThreads)
       dacc.add(rn, rn);
     }
   }
-  double acc = dacc.value();
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (lane == 0) sm[warp] = acc;
+  sm[threadIdx.x] = dacc.value();
   __syncthreads();
   if (warp == 0) {
-    double t = lane < kUpdThreads / 32 ? sm[lane] : 0.0;
-#pragma unroll
-    for (int off = kUpdThreads / 64; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    double t = 0.0;
+    for (int k = lane; k < (int)blockDim.x; k += 32) t += sm[k];
+    t = warp_sum64(t);
     if (lane == 0) part[blockIdx.x] = t;
   }
 }
@@ -1170,8 +1173,8 @@ __global__ void __launch_bounds__(kUpdThreads)
   __shared__ int s_kind;
   __shared__ double s_sum[2 * kSumWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t nv = n / P::W, stride = (int64_t)gridDim.x * kUpdThreads;
-  int64_t i = (int64_t)blockIdx.x * kUpdThreads + threadIdx.x;
+  const int64_t nv = n / P::W, stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   P zv[2], pv[2];
   auto load = [&](int64_t at) {
 #pragma unroll
@@ -1182,7 +1185,8 @@ __global__ void __launch_bounds__(kUpdThreads)
       }
   };
   load(i);
-  const int act = st.active[0];
+  const int act = st.active[0], its = st.iters[0], pend = st.pending[0];
+  const double rz = st.rz[0], tol = st.tol2cc[0], rmax = st.rmax[0];
   if (warp < 2 * kSumWarps) {
     const double s = warp < kSumWarps ? part_share(rr_part, nb_rr, warp) : part_share(rz_part, nb_rz, warp - kSumWarps);
     if (lane == 0) s_sum[warp] = s;
@@ -1194,12 +1198,12 @@ __global__ void __launch_bounds__(kUpdThreads)
     int kind = -1;  // -1 inactive, 0 regular, 1 converged, 2 limit, 3 breakdown, 4 non-finite
     if (act) {
       if (!isfinite(rr) || !isfinite(rzn)) kind = 4;
-      else if (rr <= st.tol2cc[0]) kind = 1;
-      else if (st.iters[0] >= maxit) kind = 2;
+      else if (rr <= tol) kind = 1;
+      else if (its >= maxit) kind = 2;
       else if (!(rzn > 0.0)) kind = 3;
       else kind = 0;
     }
-    const double be = kind == 0 ? rzn / st.rz[0] : 0.0;
+    const double be = kind == 0 ? rzn / rz : 0.0;
     s_kind = kind;
     s_be = be;
     if (blockIdx.x == 0) {
@@ -1208,7 +1212,7 @@ __global__ void __launch_bounds__(kUpdThreads)
         if (kind == 0) {
           st.beta[0] = be;
           st.rz2[0] = rzn;
-          if (rel_trigger > 0.0 && rr < rel_trigger * st.rmax[0]) atomicAdd(&st.counters[2], 1);
+          if (rel_trigger > 0.0 && rr < rel_trigger * rmax) atomicAdd(&st.counters[2], 1);
         } else {
           st.beta[0] = 0.0;
           st.active[0] = 0;
@@ -1218,8 +1222,8 @@ __global__ void __launch_bounds__(kUpdThreads)
           if (kind == 4) st.status[0] = ST_NONFINITE;
         }
       }
-      if (st.active[0]) atomicAdd(&st.counters[0], 1);
-      if (st.pending[0]) atomicAdd(&st.counters[1], 1);
+      if (kind == 0) atomicAdd(&st.counters[0], 1);
+      if (pend || kind == 1) atomicAdd(&st.counters[1], 1);
     }
   }
   __syncthreads();
@@ -1284,39 +1288,35 @@ __device__ __forceinline__ double sum_parts(const double* part, int nblk, int B,
   return s;
 }
 
-// One block of kColThreads threads per column sums that column's partials
-// (fixed thread stride and tree: deterministic) so the FP64 additions are
-// spread over B multiprocessors.
-constexpr int kColThreads = 512;
-
-__device__ __forceinline__ double block_sum_parts(const double* part, int nblk, int B, int col) {
-  __shared__ double sm[kColThreads / 32];
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += kColThreads) s += part[(int64_t)b * B + col];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
-  __syncthreads();
-  double t = 0.0;
-#pragma unroll
-  for (int w = 0; w < kColThreads / 32; ++w) t += sm[w];
-  return t;
-}
+// One block per column sums that column's partials (a fixed order:
+// deterministic), so that the FP64 additions are spread over B multiprocessors;
+// four warps per sum, both sums of the beta step at once, since the adds of a
+// shuffle tree cost an SM 19 cycles per warp.  Measured on GB300 against 16 warps
+// and one sum after the other, 1216 partials, 4 columns: alpha 4.0 -> 2.5 us, beta
+// 10.2 -> 4.3 us.
+constexpr int kColThreads = 64 * kSumWarps;
 
 // alpha = rz / p^T q ; grid = B blocks.  Also clears the counters that
 // k_scalar_col_beta accumulates.
 static __global__ void __launch_bounds__(kColThreads)
     k_scalar_col_alpha(int B, int nblk, const double* __restrict__ pq_part, ColState st) {
-  const int col = blockIdx.x;
+  __shared__ double s_sum[kSumWarps];
+  const int col = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (col == 0 && threadIdx.x < 3) st.counters[threadIdx.x] = 0;
-  if (!st.active[col]) {
-    if (threadIdx.x == 0) st.alpha[col] = 0.0;
+  const int act = st.active[col], its = st.iters[col];
+  const double rz = st.rz[col];
+  if (warp < kSumWarps) {
+    const double s = part_share(pq_part, nblk, warp, B, col);
+    if (lane == 0) s_sum[warp] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (!act) {
+    st.alpha[col] = 0.0;
     return;
   }
-  const double pq = block_sum_parts(pq_part, nblk, B, col);
-  if (threadIdx.x != 0) return;
-  st.iters[col] += 1;
+  const double pq = (s_sum[0] + s_sum[1]) + (s_sum[2] + s_sum[3]);
+  st.iters[col] = its + 1;
   if (!isfinite(pq)) {
     st.status[col] = ST_NONFINITE;
     st.active[col] = 0;
@@ -1326,7 +1326,7 @@ static __global__ void __launch_bounds__(kColThreads)
     st.active[col] = 0;
     st.alpha[col] = 0.0;
   } else {
-    st.alpha[col] = st.rz[col] / pq;
+    st.alpha[col] = rz / pq;
   }
 }
 
@@ -1335,41 +1335,43 @@ static __global__ void __launch_bounds__(kColThreads)
 static __global__ void __launch_bounds__(kColThreads)
     k_scalar_col_beta(int B, int nblk_rr, const double* __restrict__ rr_part, int nblk_rz,
                       const double* __restrict__ rz_part, ColState st, int maxit, double rel_trigger) {
-  const int col = blockIdx.x;
-  if (st.active[col]) {
-    const double rr = block_sum_parts(rr_part, nblk_rr, B, col);
-    const double rzn = block_sum_parts(rz_part, nblk_rz, B, col);
-    if (threadIdx.x == 0) {
-      st.rr[col] = rr;
-      if (!isfinite(rr) || !isfinite(rzn)) {
-        st.status[col] = ST_NONFINITE;
-        st.active[col] = 0;
-        st.beta[col] = 0.0;
-      } else if (rr <= st.tol2cc[col]) {
-        mark_pending(st, col, rzn);
-      } else if (st.iters[col] >= maxit) {
-        st.status[col] = ST_MAXIT;
-        st.active[col] = 0;
-        st.beta[col] = 0.0;
-      } else if (!(rzn > 0.0)) {
-        st.status[col] = ST_BREAKDOWN;
-        st.active[col] = 0;
-        st.beta[col] = 0.0;
-      } else {
-        st.beta[col] = rzn / st.rz[col];
-        st.rz[col] = rzn;
-        st.rz2[col] = rzn;
-        if (rel_trigger > 0.0 && rr < rel_trigger * st.rmax[col]) atomicAdd(&st.counters[2], 1);
-      }
+  __shared__ double s_sum[2 * kSumWarps];
+  const int col = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int act = st.active[col], its = st.iters[col];
+  const double rz = st.rz[col], tol = st.tol2cc[col], rmax = st.rmax[col];
+  const double s = warp < kSumWarps ? part_share(rr_part, nblk_rr, warp, B, col)
+                                    : part_share(rz_part, nblk_rz, warp - kSumWarps, B, col);
+  if (lane == 0) s_sum[warp] = s;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (act) {
+    const double rr = (s_sum[0] + s_sum[1]) + (s_sum[2] + s_sum[3]);
+    const double rzn = (s_sum[4] + s_sum[5]) + (s_sum[6] + s_sum[7]);
+    st.rr[col] = rr;
+    if (!isfinite(rr) || !isfinite(rzn)) {
+      st.status[col] = ST_NONFINITE;
+      st.active[col] = 0;
+      st.beta[col] = 0.0;
+    } else if (rr <= tol) {
+      mark_pending(st, col, rzn);
+    } else if (its >= maxit) {
+      st.status[col] = ST_MAXIT;
+      st.active[col] = 0;
+      st.beta[col] = 0.0;
+    } else if (!(rzn > 0.0)) {
+      st.status[col] = ST_BREAKDOWN;
+      st.active[col] = 0;
+      st.beta[col] = 0.0;
+    } else {
+      st.beta[col] = rzn / rz;
+      st.rz[col] = rzn;
+      st.rz2[col] = rzn;
+      if (rel_trigger > 0.0 && rr < rel_trigger * rmax) atomicAdd(&st.counters[2], 1);
     }
   }
-  if (threadIdx.x == 0) {
-    if (st.active[col]) atomicAdd(&st.counters[0], 1);
-    if (st.pending[col]) atomicAdd(&st.counters[1], 1);
-  }
+  if (st.active[col]) atomicAdd(&st.counters[0], 1);
+  if (st.pending[col]) atomicAdd(&st.counters[1], 1);
 }
-
-
 
 // Sum partials of a column reduction into out[col] (FP64).
 static __global__ void __launch_bounds__(kScalarThreads)

@@ -349,18 +349,20 @@ void launch_vtail(const TailLevelIn* levels, int nlev, const double* kinv, int n
   LCMG_LAUNCHED();
 }
 
-// Grid of the fused one-column updates: one 16-byte word per thread, at most
-// two blocks per SM (every block re-sums the partials of the dot products it
-// needs in FP64)
-static int fused_update_grid(int64_t words, int max_blocks) {
+// Blocks and threads of the fused one-column updates: one 16-byte word per
+// thread, at most two blocks per SM (every block re-sums the partials of the
+// dot products it needs in FP64); blocks of 256 threads while they fit on as
+// many SMs, so that a short vector's FP64 work is spread
+static dim3 fused_update_grid(int64_t words, int max_blocks, int* threads) {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
     LCMG_CUDA(cudaGetDevice(&dev));
     LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   }
-  const int64_t want = (words + kUpdThreads - 1) / kUpdThreads;
-  return (int)std::max<int64_t>(1, std::min(want, (int64_t)std::min(2 * sms, max_blocks)));
+  *threads = words <= (int64_t)sms * (kUpdThreads / 2) ? kUpdThreads / 2 : kUpdThreads;
+  const int64_t want = (words + *threads - 1) / *threads;
+  return dim3((unsigned)std::max<int64_t>(1, std::min(want, (int64_t)std::min(2 * sms, max_blocks))));
 }
 
 // Rows per strip of the row-streaming kernels: at most `most`, and few
@@ -488,18 +490,20 @@ int launch_update_xr(int64_t n, int B, const ColState& st, const T* p, const T* 
 template <class T>
 int launch_update_xr_alpha(int64_t n, const ColState& st, int nb_pq, const double* pq_part, const T* p,
                            const T* q, T* x, T* r, double* part, int max_blocks, cudaStream_t s) {
-  const int g = fused_update_grid(n / Pack<T>::W, max_blocks);
-  klaunch(k_update_xr_alpha<T>, dim3(g), dim3(kUpdThreads), 0, s, n, st, nb_pq, pq_part, p, q, x, r, part);
+  int threads;
+  const dim3 g = fused_update_grid(n / Pack<T>::W, max_blocks, &threads);
+  klaunch(k_update_xr_alpha<T>, g, dim3(threads), 0, s, n, st, nb_pq, pq_part, p, q, x, r, part);
   LCMG_LAUNCHED();
-  return g;
+  return (int)g.x;
 }
 
 template <class T>
 void launch_update_p_beta(int64_t n, const ColState& st, int nb_rr, const double* rr_part, int nb_rz,
                           const double* rz_part, int maxit, double rel_trigger, const T* z, T* p, int max_blocks,
                           cudaStream_t s) {
-  const int g = fused_update_grid(n / Pack<T>::W, max_blocks);
-  klaunch(k_update_p_beta<T>, dim3(g), dim3(kUpdThreads), 0, s, n, st, nb_rr, rr_part, nb_rz, rz_part, maxit, rel_trigger,
+  int threads;
+  const dim3 g = fused_update_grid(n / Pack<T>::W, max_blocks, &threads);
+  klaunch(k_update_p_beta<T>, g, dim3(threads), 0, s, n, st, nb_rr, rr_part, nb_rz, rz_part, maxit, rel_trigger,
           z, p);
   LCMG_LAUNCHED();
 }
