@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "launch.h"
+#include "psf_tile.cuh"
 #include "vfused.cuh"
 #include "paper_mg.cuh"
 #include "rs_amg.h"
@@ -1049,13 +1050,19 @@ int Batch<T>::apply_K(const T* P, T* Q, double* part) {
                                            part, c.maxblk, s);
   } else {
     // PSF operator
-    nb = grid_for(c.n, B, c.maxblk);
     PsfArgs pa = psf();
-    klaunch(k_psf_forward<T, 0>, dim3(nb), dim3(kBlock), 0, s, pa, psfT(), B, P, Y, nullptr, 1, 1, nullptr);
-    LCMG_LAUNCHED();
-    mark();
-    klaunch(k_psf_normal<T, T, 1>, dim3(nb), dim3(kBlock), 0, s, pa, psfT(), B, Y, fop(), P, nullptr, c.lam2.p, Q, part);
-    LCMG_LAUNCHED();
+    if constexpr (std::is_same<T, float>::value) {
+      launch_psf<0, PSF_STORE>(pa, psfT(), B, P, Y, fop(), nullptr, nullptr, nullptr, c.maxblk, s);
+      mark();
+      nb = launch_psf<1, PSF_NORMAL>(pa, psfT(), B, Y, Q, fop(), P, c.lam2.p, part, c.maxblk, s);
+    } else {
+      nb = grid_for(c.n, B, c.maxblk);
+      klaunch(k_psf_forward<T, 0>, dim3(nb), dim3(kBlock), 0, s, pa, psfT(), B, P, Y, nullptr, 1, 1, nullptr);
+      LCMG_LAUNCHED();
+      mark();
+      klaunch(k_psf_normal<T, T, 1>, dim3(nb), dim3(kBlock), 0, s, pa, psfT(), B, Y, fop(), P, nullptr, c.lam2.p, Q, part);
+      LCMG_LAUNCHED();
+    }
   }
   mark();
   return nb;

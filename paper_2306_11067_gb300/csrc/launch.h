@@ -123,6 +123,14 @@ template <class T>
 void launch_copy_cols(int64_t n, int B, const int* flag, const T* src, T* dst, int max_blocks,
                       cudaStream_t s);
 
+// ---- blur without 1-D factors, FP32 (separable.cu, psf_tile.cuh) ------------
+// out = A in (TRANS 0, PSF_STORE) or A^T in + lam2 L^T W L P with the partials
+// of P.out (TRANS 1, PSF_NORMAL); returns the block count (rows of the
+// partial sums)
+template <int TRANS, int EPI>
+int launch_psf(const PsfArgs& a, const float* psf, int B, const float* in, float* out, const FineOp<float>& fop,
+               const float* P, const double* lam2, double* part, int max_blocks, cudaStream_t s);
+
 // ---- separable blur (separable.cu) ----------------------------------------
 // One banded 1-D pass in FP64 as built on the host: out(o) = sum_k
 // c[k] in(o - H + k), plus the correction rows d of the first nlo and the

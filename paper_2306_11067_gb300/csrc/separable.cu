@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "launch.h"
+#include "psf_tile.cuh"
 #include "separable.cuh"
 
 namespace lcmg {
@@ -243,6 +244,32 @@ int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, 
   return band_direct<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
 }
 
+// Tiles of 8 rows in blocks of 64 threads while that leaves SMs idle, else of
+// 32 rows (the halo of 2 rh rows is staged per tile); one output per thread
+// where the PSF's tile does not fit in kPsfSmem (radii above 24 or so).
+template <int TRANS, int EPI>
+int launch_psf(const PsfArgs& a, const float* psf, int B, const float* in, float* out, const FineOp<float>& fop,
+               const float* P, const double* lam2, double* part, int max_blocks, cudaStream_t s) {
+  const int nti = (a.nv + kPsfTI - 1) / kPsfTI;
+  auto tiles = [&](int tj) { return (int64_t)nti * ((a.nh + tj - 1) / tj); };
+  const int tj = tiles(32) * B < 304 || psf_smem(a.rv, a.rh, 32) > kPsfSmem ? 8 : 32;
+  const size_t smem = psf_smem(a.rv, a.rh, tj);
+  if (smem <= kPsfSmem) {
+    const int blocks = clamp_blocks(tiles(tj), max_blocks);
+    klaunch(k_psf_tile<TRANS, EPI>, dim3((unsigned)blocks, (unsigned)B), dim3(8 * tj), smem, s, a, psf, B, in, out, fop, P,
+            lam2, part);
+    LCMG_LAUNCHED();
+    return blocks;
+  }
+  const int g = grid_for((int64_t)a.nv * a.nh, B, max_blocks);
+  if constexpr (EPI == PSF_STORE)
+    klaunch(k_psf_forward<float, 0>, dim3(g), dim3(kBlock), 0, s, a, psf, B, in, out, nullptr, 1, 1, nullptr);
+  else
+    klaunch(k_psf_normal<float, float, 1>, dim3(g), dim3(kBlock), 0, s, a, psf, B, in, fop, P, nullptr, lam2, out, part);
+  LCMG_LAUNCHED();
+  return g;
+}
+
 void launch_sep_diag(int nv, int nh, const double* dv, const double* dh, double* diag, int max_blocks,
                      cudaStream_t s) {
   const int64_t n = (int64_t)nv * nh;
@@ -265,5 +292,10 @@ LCMG_BAND_INST(double, double, 1, BAND_NORMAL)
 LCMG_BAND_INST(double, double, 1, BAND_RESID2)
 LCMG_BAND_INST(double, double, 1, BAND_TRUERES)
 #undef LCMG_BAND_INST
+
+template int launch_psf<0, PSF_STORE>(const PsfArgs&, const float*, int, const float*, float*, const FineOp<float>&,
+                                      const float*, const double*, double*, int, cudaStream_t);
+template int launch_psf<1, PSF_NORMAL>(const PsfArgs&, const float*, int, const float*, float*, const FineOp<float>&,
+                                       const float*, const double*, double*, int, cudaStream_t);
 
 }  // namespace lcmg

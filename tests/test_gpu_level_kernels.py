@@ -51,3 +51,31 @@ def test_cycle_in_strips_matches_its_model(n_v, n_h, levels, cols, smoother):
         ref = V(R[k])
         assert np.linalg.norm(zd[k].cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
     s.close()
+
+
+@pytest.mark.parametrize("n_v,n_h,kv,kh", [
+    (40, 36, 1, 4),     # 3 and 9 taps: words of taps with a remainder of three and one
+    (72, 56, 7, 7),     # ragged tiles
+    (33, 27, 5, 2),     # one level
+    (80, 96, 34, 34),   # too large for the tiles: one output per thread
+    (640, 512, 2, 3),   # tiles of 32 rows
+])
+def test_mixed_blur_follows_fp64(n_v, n_h, kv, kh):
+    rng = pg.rng(5)
+    u, v = np.arange(-kv, kv + 1)[:, None], np.arange(-kh, kh + 1)[None, :]
+    psf = np.exp(-(0.8 * u + 0.6 * v) ** 2 / 9.0 - (0.8 * v - 0.6 * u) ** 2 / 2.0) * rng.uniform(0.7, 1.3, (2 * kv + 1, 2 * kh + 1))
+    psf /= psf.sum()
+    d = pg.random_weights(ops.n_edges(n_v, n_h), 4, d_min=0.05)
+    b = rng.standard_normal((1, n_v * n_h)) + 1.0
+    got = {}
+    for prec in (L.PREC_FP64, L.PREC_MIXED):
+        s = Solver(n_v, n_h, precision=prec, tol=1e-11, maxit=5000)
+        s.set_forward_stencil(psf)
+        assert s.forward_form() == L.FORM_PSF2D
+        s.set_weights(d)
+        got[prec] = s.solve(np.array([0.5]), b)
+        s.close()
+    a, m = got[L.PREC_FP64], got[L.PREC_MIXED]
+    assert a["status"][0, 0] == 0 and m["status"][0, 0] == 0
+    assert np.linalg.norm(m["x"] - a["x"]) <= 1e-6 * np.linalg.norm(a["x"])
+    assert m["iters"][0, 0] <= 1.15 * a["iters"][0, 0] + 12, (a["iters"], m["iters"])
