@@ -362,15 +362,19 @@ static void build_hierarchy(lcmg_ctx& c) {
     double* ga = g.ga.need(kStencil * g.n);
     RapIn in{};
     in.nvf = f.nv; in.nhf = f.nh; in.nf = f.n;
+    RapIn in2 = in;
     if (k == 1) {
-      in.ws = c.ws.p; in.we = c.we.p; in.ga = c.diag.p;
-      in.part = 0; launch_galerkin(in, g.nv, g.nh, gl, c.maxblk, c.stream);
-      in.part = 1; launch_galerkin(in, g.nv, g.nh, ga, c.maxblk, c.stream);
+      in.ws = in2.ws = c.ws.p;
+      in.we = in2.we = c.we.p;
+      in.ga = in2.ga = c.diag.p;
+      in.part = 0;
+      in2.part = 1;
     } else {
-      in.part = 2;
-      in.g25 = f.gl.p; launch_galerkin(in, g.nv, g.nh, gl, c.maxblk, c.stream);
-      in.g25 = f.ga.p; launch_galerkin(in, g.nv, g.nh, ga, c.maxblk, c.stream);
+      in.part = in2.part = 2;
+      in.g25 = f.gl.p;
+      in2.g25 = f.ga.p;
     }
+    launch_galerkin(in, in2, g.nv, g.nh, gl, ga, c.stream);
     // smoother copies: per-point rows of both parts (FP64 and FP32)
     const int gg = (int)std::min<int64_t>((kCoefStride * g.n + kBlock - 1) / kBlock, c.maxblk);
     klaunch(k_coef_pack<double>, dim3(gg), dim3(kBlock), 0, c.stream, g.n, gl, ga, g.cf64.need(kCoefStride * g.n));

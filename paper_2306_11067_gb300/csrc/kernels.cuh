@@ -895,8 +895,7 @@ static __global__ void __launch_bounds__(4 * kInvTile * kInvTile)
 }
 
 // ---------------------------------------------------------------------------
-// Galerkin coarse operators G_c = P^T G_f P (Sec. 3.1), one thread per
-// (coarse point, stencil offset).  The fine operator is either the level-0
+// Galerkin coarse operators G_c = P^T G_f P (Sec. 3.1).  The fine operator is either the level-0
 // 5-point L^T W L (part 0), the level-0 diagonal diag(A^T A) (part 1), or a
 // 25-point coarse stencil (part 2).
 // ---------------------------------------------------------------------------
@@ -928,43 +927,104 @@ struct RapIn {
   }
 };
 
-static __global__ void __launch_bounds__(kBlock) k_galerkin(RapIn in, int nvc, int nhc, double* __restrict__ out) {
-  const int64_t nc = (int64_t)nvc * nhc;
-  const int R = (in.part == 2) ? 2 : 1;
-  for (int64_t t = (int64_t)blockIdx.x * kBlock + threadIdx.x; t < nc * kStencil;
-       t += (int64_t)gridDim.x * kBlock) {
-    const int o = (int)(t / nc);
-    const int64_t P = t - (int64_t)o * nc;
-    const int J = (int)(P / nvc), I = (int)(P - (int64_t)J * nvc);
-    const int oi = o % 5 - 2, oj = o / 5 - 2;
-    const int It = I + oi, Jt = J + oj;
-    double sum = 0.0;
-    if (It >= 0 && It < nvc && Jt >= 0 && Jt < nhc) {
-      for (int b = 2 * J - 1; b <= 2 * J + 2; ++b) {
-        if (b < 0 || b >= in.nhf) continue;
-        const double wb = pw1(b, J, nhc);
-        for (int a = 2 * I - 1; a <= 2 * I + 2; ++a) {
-          if (a < 0 || a >= in.nvf) continue;
-          const double wab = wb * pw1(a, I, nvc);
-          const int64_t f = (int64_t)a + (int64_t)b * in.nvf;
-          for (int dj = -R; dj <= R; ++dj) {
-            const int d = b + dj;
-            if (d < 0 || d >= in.nhf) continue;
-            const double wd = pw1(d, Jt, nhc);
-            if (wd == 0.0) continue;
-            for (int di = -R; di <= R; ++di) {
-              const int c = a + di;
-              if (c < 0 || c >= in.nvf) continue;
-              if (in.part != 2 && di != 0 && dj != 0) continue;
-              const double wc = pw1(c, It, nvc);
-              if (wc == 0.0) continue;
-              sum += wab * in.coef(di, dj, f, a, b) * wc * wd;
-            }
-          }
-        }
-      }
+// P^T G P is contracted along i first, H(b, dj, I) = sum_{a, di} w(a, I)
+// w(a + di, I + oi) G(di, dj; a, b) for the fine rows b of a tile of 32 x 2
+// coarse points, and then along j from shared memory.  A block takes one of
+// the five oi (blockIdx.y) of one of two operators on the same grid
+// (blockIdx.z).
+//
+// What bounds it: the FP64 pipe (about 500 multiply-adds per us on the GPU,
+// 19 cycles per warp instruction on an SM), so the two contractions take
+// some 700 multiply-adds per coarse point where the product over all pairs of
+// fine points took 1600 terms of four operations; on small levels one block's
+// chain, so the oi are separate blocks.  Measured on GB300, both operators of
+// a level, against one thread per (coarse point, offset): 256 x 160 coarse
+// points (5-point fine operator) 322 -> 100 us, 128 x 80 274 -> 42 us, 64 x 40 152 ->
+// 16 us.
+constexpr int kGalTJ = 2;                           // coarse rows per tile
+constexpr int kGalThreads = 32 * (2 * kGalTJ + 2);  // a warp per fine row
+
+// The weight of fine point 2I - 1 + q in coarse point I of nc is 1/4, 3/4 or 1;
+// gal_k tells which (0, 1, 2) and sW[3 a + b] holds the products of two (a
+// table, so that no FP64 operation goes into weights)
+__device__ __forceinline__ int gal_k(int q, int I, int nc) {
+  return q == 1 ? (I == 0 ? 2 : 1) : q == 2 ? (I == nc - 1 ? 2 : 1) : 0;
+}
+
+// H of fine row b (|dj| <= R) for I: sH[dj + 2][lane]
+template <int OI>
+__device__ __forceinline__ void gal_row(const RapIn& in, int R, int I, int nvc, int b, const double* sW,
+                                        double (*sH)[32], int lane) {
+  const bool ok = I < nvc && I + OI >= 0 && I + OI < nvc && b >= 0 && b < in.nhf;
+  double w[4][4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      constexpr int kShift = 2 * OI;
+      if (kShift + q - m >= -2 && kShift + q - m <= 2) w[m][q] = sW[3 * gal_k(m, I, nvc) + gal_k(q, I + OI, nvc)];
     }
-    out[t] = sum;
+  for (int dj = -R; dj <= R; ++dj) {
+    double h = 0.0;
+    if (ok && b + dj >= 0 && b + dj < in.nhf) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          constexpr int kShift = 2 * OI;
+          const int di = kShift + q - m;  // from fine point m of I to fine point q of I + OI
+          if (di < -2 || di > 2) continue;
+          if (in.part != 2 && ((di != 0 && dj != 0) || di < -R || di > R)) continue;
+          const int a = 2 * I - 1 + m;
+          if (a < 0 || a >= in.nvf || a + di < 0 || a + di >= in.nvf) continue;
+          h += w[m][q] * in.coef(di, dj, (int64_t)a + (int64_t)b * in.nvf, a, b);
+        }
+    }
+    sH[dj + 2][lane] = h;
+  }
+}
+
+static __global__ void __launch_bounds__(kGalThreads)
+    k_galerkin(RapIn in0, RapIn in1, int nvc, int nhc, double* __restrict__ out0, double* __restrict__ out1) {
+  __shared__ double sH[2 * kGalTJ + 2][5][32];  // [fine row][dj][I]
+  __shared__ double sW[9];
+  if (threadIdx.x < 9) {
+    const int a = threadIdx.x / 3, b = threadIdx.x % 3;
+    sW[threadIdx.x] = (a == 0 ? 0.25 : a == 1 ? 0.75 : 1.0) * (b == 0 ? 0.25 : b == 1 ? 0.75 : 1.0);
+  }
+  __syncthreads();
+  const RapIn& in = blockIdx.z == 0 ? in0 : in1;
+  double* __restrict__ out = blockIdx.z == 0 ? out0 : out1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nti = (nvc + 31) / 32, oi = (int)blockIdx.y - 2;
+  const int I = (int)blockIdx.x % nti * 32 + lane, J0 = (int)blockIdx.x / nti * kGalTJ;
+  const int R = in.part == 2 ? 2 : in.part == 0 ? 1 : 0;  // |dj| <= R
+  const int64_t nc = (int64_t)nvc * nhc;
+  const int b = 2 * J0 - 1 + w;  // along i: warp w takes fine row b
+  switch (oi) {
+    case -2: gal_row<-2>(in, R, I, nvc, b, sW, sH[w], lane); break;
+    case -1: gal_row<-1>(in, R, I, nvc, b, sW, sH[w], lane); break;
+    case 0: gal_row<0>(in, R, I, nvc, b, sW, sH[w], lane); break;
+    case 1: gal_row<1>(in, R, I, nvc, b, sW, sH[w], lane); break;
+    default: gal_row<2>(in, R, I, nvc, b, sW, sH[w], lane); break;
+  }
+  __syncthreads();
+  // along j: the warps share (coarse row, oj)
+  for (int task = w; task < 5 * kGalTJ; task += kGalThreads / 32) {
+    const int Jl = task / 5, oj = task - 5 * Jl - 2, J = J0 + Jl;
+    if (I >= nvc || J >= nhc) continue;
+    double g = 0.0;
+    if (I + oi >= 0 && I + oi < nvc && J + oj >= 0 && J + oj < nhc) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int dj = 2 * oj + q - m;
+          if (dj < -R || dj > R) continue;
+          g += sW[3 * gal_k(m, J, nhc) + gal_k(q, J + oj, nhc)] * sH[2 * Jl + m][dj + 2][lane];
+        }
+    }
+    out[(int64_t)((oi + 2) + 5 * (oj + 2)) * nc + (int64_t)J * nvc + I] = g;
   }
 }
 

@@ -470,11 +470,9 @@ void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, i
   }
 }
 
-void launch_galerkin(const RapIn& in, int nvc, int nhc, double* out, int max_blocks, cudaStream_t s) {
-  const int64_t work = (int64_t)nvc * nhc * kStencil;
-  int64_t g = (work + kBlock - 1) / kBlock;
-  if (g > max_blocks) g = max_blocks;
-  klaunch(k_galerkin, dim3((unsigned)g), dim3(kBlock), 0, s, in, nvc, nhc, out);
+void launch_galerkin(const RapIn& in0, const RapIn& in1, int nvc, int nhc, double* out0, double* out1, cudaStream_t s) {
+  const unsigned tiles = (unsigned)((nvc + 31) / 32) * (unsigned)((nhc + kGalTJ - 1) / kGalTJ);
+  klaunch(k_galerkin, dim3(tiles, 5, 2), dim3(kGalThreads), 0, s, in0, in1, nvc, nhc, out0, out1);
   LCMG_LAUNCHED();
 }
 

@@ -53,6 +53,33 @@ def test_cycle_in_strips_matches_its_model(n_v, n_h, levels, cols, smoother):
     s.close()
 
 
+@pytest.mark.parametrize("n_v,n_h,levels", [(140, 72, 3), (12, 10, 2), (4, 130, 2), (256, 6, 2)])
+def test_galerkin_tiles(n_v, n_h, levels):
+    s = Solver(n_v, n_h, levels=levels)
+    s.set_forward_stencil(pg.gaussian_psf(2, 1.0))
+    d = pg.random_weights(ops.n_edges(n_v, n_h), 5, d_min=0.05)
+    s.set_weights(d)
+    z = torch.zeros(1, n_v * n_h, device="cuda", dtype=torch.float64)
+    L.lcmg_apply_vcycle_dev(s.ctx, np.array([0.3]), z, torch.empty_like(z))  # builds the hierarchy
+    diag = L.lcmg_get_diag(s.ctx, n_v * n_h)
+    H = mg.build_hierarchy(mg.weighted_laplacian(ops.gradient(n_v, n_h), d), sp.diags(diag), n_v, n_h, levels)
+    for k in range(1, levels):
+        nv, nh, gl, ga = L.lcmg_get_level(s.ctx, k)
+        for got, ref in ((gl, H.G_L[k]), (ga, H.G_A[k])):
+            ref = ref.tocsr()
+            n = nv * nh
+            i, j = np.arange(n) % nv, np.arange(n) // nv
+            acc = sp.csr_matrix((n, n))
+            for o in range(25):
+                di, dj = o % 5 - 2, o // 5 - 2
+                ok = (i + di >= 0) & (i + di < nv) & (j + dj >= 0) & (j + dj < nh)
+                assert (np.asarray(got[o])[~ok] == 0).all()
+                p = np.arange(n)[ok]
+                acc = acc + sp.csr_matrix((np.asarray(got[o])[ok], (p, p + di + dj * nv)), shape=(n, n))
+            assert abs(acc - ref).max() <= 1e-13 * abs(ref).max()
+    s.close()
+
+
 @pytest.mark.parametrize("n_v,n_h,kv,kh", [
     (40, 36, 1, 4),     # 3 and 9 taps: words of taps with a remainder of three and one
     (72, 56, 7, 7),     # ragged tiles
