@@ -434,7 +434,7 @@ static void ensure_work(lcmg_ctx& c, int B) {
     if (k > 0) { c.lw[k].rhs.need(nk); c.lw[k].z.need(nk); }
   }
   const size_t nc = (size_t)c.lev[L - 1].n;
-  c.kinv.need(nc * nc * B); c.Mw.need(nc * nc * B); c.Ww.need(nc * nc * B);
+  c.kinv.need(nc * nc * B); c.Mw.need(nc * nc * B); c.Ww.need(dense_inverse_scratch(nc) * B);
   c.lam2.need(B); c.lam2T.need(B * tb);
   const size_t pb = (size_t)kMaxBlocks * B;
   c.part_pq.need(pb); c.part_rr.need(pb); c.part_rz.need(pb); c.part_x.need(pb);
@@ -1254,7 +1254,7 @@ static void alloc_pm_work(lcmg_ctx& c, const std::vector<int64_t>& sizes) {
     }
   }
   const size_t nc = (size_t)sizes[L - 1];
-  c.kinv.need(nc * nc); c.Mw.need(nc * nc); c.Ww.need(nc * nc);
+  c.kinv.need(nc * nc); c.Mw.need(nc * nc); c.Ww.need(dense_inverse_scratch(nc));
 }
 
 template <class I>

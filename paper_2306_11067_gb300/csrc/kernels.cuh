@@ -774,22 +774,24 @@ __global__ void __launch_bounds__(kBlock)
 // of S_kj.  Every element sees the additions of the unblocked algorithm in
 // its order (increasing k), so the result does not depend on the tiling.
 //
-// What bounds it: FP64 runs at less than two multiply-adds per clock and SM
-// here, so the n^3 / 2 of them have to be spread over the GPU: one block of
-// threads per 16 x 16 tile (136 at n = 256), one launch per step; and the
-// chain of 16 dependent pivots (square root and reciprocal, about 80 cycles
-// per FP64 operation), which every block goes through again for the pivot
-// block rather than wait for another launch.  So that little else stands in
-// the chain, the pivot block, the two panels and the tile have 256 threads
-// each, a column's threads lie in different SM quarters for the three
-// solves, and a division is three operations from the pivot's reciprocal.
-// A step reads `src` and writes `dst` (the pivot row and column are read by
-// every block).  info[col] = the 1-based index of the first pivot that was
-// not positive.
+// A step is two launches: k_inverse_panel solves the panel of every block row
+// (one block each, which goes through the pivot block's 16 dependent pivots
+// itself rather than wait for a third launch) and k_inverse_update advances
+// every tile with two of the panels.
 //
-// Measured on GB300 against one block per column that did all of it in
-// global memory: n = 160 2,530 -> 187 us, n = 256 11,400 -> about 300 us,
-// n = 567 123,000 -> 2,220 us; the same values bit for bit.
+// What bounds it: the chain of pivots (square root and reciprocal, about 80
+// cycles per FP64 operation) at small n, so little else stands in it: the
+// pivot block and the panel have 256 threads each, a column's threads lie in
+// different SM quarters for the two solves, and a division is three
+// operations from the pivot's reciprocal; at large n the FP64 pipe (less than
+// two multiply-adds per clock and SM) of the updates.  A step reads `src` and
+// writes `dst` (the pivot row and column are read by every panel).
+// info[col] = the 1-based index of the first pivot that was not positive.
+//
+// Measured on GB300, per step, against one launch whose every tile solved
+// both of its panels again: n = 256 18.7 -> 15.4 + 2.8 us, n = 567 61 -> 15.5 + 7.2 us.
+// (One block per column that did all of it in
+// global memory took 123 ms at n = 567; the values are the same bit for bit.)
 constexpr int kInvTile = 16;
 
 // sqrt(a) and its reciprocal, both rounded to nearest: an FP32 seed, one
@@ -810,46 +812,39 @@ __device__ __forceinline__ void pivot_root(double a, double& root, double& recip
   }
 }
 
-static __global__ void __launch_bounds__(4 * kInvTile * kInvTile)
-    k_inverse_step(int n, int k, int last, const double* __restrict__ srcall, double* __restrict__ dstall,
-                   int* __restrict__ info) {
+// element (rr, cc) of tile (u, v), u >= v; a last partial tile is padded with
+// the rows and columns of the identity
+__device__ __forceinline__ double inverse_get(const double* __restrict__ S, int n, int u, int v, int rr, int cc) {
+  const int i = u * kInvTile + rr, j = v * kInvTile + cc;
+  if (i < n && j < n) return S[(int64_t)i * n + j];
+  return i == j ? 1.0 : 0.0;
+}
+
+static __global__ void __launch_bounds__(2 * kInvTile * kInvTile)
+    k_inverse_panel(int n, int k, const double* __restrict__ srcall, double* __restrict__ panall,
+                    int* __restrict__ info) {
   constexpr int Q = kInvTile;
-  // the pivot block (then its factor, lower triangle) and the two panels
-  __shared__ double A[3][Q][Q + 1];
+  // the pivot block (then its factor, lower triangle) and the panel
+  __shared__ double A[2][Q][Q + 1];
   __shared__ double s_piv, s_rec;
   __shared__ int bad;
-  const int col = blockIdx.y;
+  const int col = blockIdx.y, b = blockIdx.x;
   const double* __restrict__ S = srcall + (int64_t)col * n * n;
-  double* __restrict__ O = dstall + (int64_t)col * n * n;
-  // tile (bi, bj), bi >= bj, of the lower triangle
-  int bi = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
-  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
-  while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
-  const int bj = (int)blockIdx.x - bi * (bi + 1) / 2;
-  // group 0: pivot block, 1 and 2: panels of block rows bi and bj, 3: tile;
-  // a half warp holds a column, the groups' columns shifted by one warp
+  // group 0: pivot block, 1: the panel of block row b; a half warp holds a
+  // column, the groups' columns shifted by one warp
   const int g = threadIdx.x / (Q * Q), l = threadIdx.x % (Q * Q);
   const int c = 2 * ((l / 32 + 8 - g) % 8) + (l / 16) % 2, r = l % Q;
-  // element (rr, cc) of tile (u, v), u >= v; a last partial tile is padded
-  // with the rows and columns of the identity
-  auto get = [&](int u, int v, int rr, int cc) {
-    const int i = u * Q + rr, j = v * Q + cc;
-    if (i < n && j < n) return S[(int64_t)i * n + j];
-    return i == j ? 1.0 : 0.0;
-  };
-  // the panel of block row b: rows of M_bk (b > k), the identity (b = k), or
-  // the columns of S_kb (b < k)
-  auto panel = [&](int b, int rr, int cc) {
-    if (b > k) return get(b, k, rr, cc);
-    if (b == k) return rr == cc ? 1.0 : 0.0;
-    return get(k, b, cc, rr);
-  };
-  const bool trail = bi > k;  // the tile subtracts (else it adds)
-  double x = g == 0   ? get(k, k, r, c)
-             : g == 1 ? panel(bi, r, c)
-             : g == 2 ? panel(bj, r, c)
-             : (trail ? bj == k : bi == k) ? 0.0
-                                           : get(bi, bj, r, c);
+  auto get = [&](int u, int v, int rr, int cc) { return inverse_get(S, n, u, v, rr, cc); };
+  double x;
+  if (g == 0) {
+    x = get(k, k, r, c);
+  } else if (b > k) {  // rows of M_bk
+    x = get(b, k, r, c);
+  } else if (b == k) {  // the identity
+    x = r == c ? 1.0 : 0.0;
+  } else {  // the columns of S_kb
+    x = get(k, b, c, r);
+  }
   auto pivot = [&](int t, double a) {
     if (!(a > 0.0)) {
       if (!bad) bad = k * Q + t + 1;
@@ -866,7 +861,7 @@ static __global__ void __launch_bounds__(4 * kInvTile * kInvTile)
   }
   __syncthreads();
   for (int t = 0; t < Q; ++t) {
-    if (c == t && g < 3) {  // column t, final
+    if (c == t) {  // column t, final
       const double piv = s_piv, rec = s_rec;
       if (g == 0 && r == t) {
         x = piv;
@@ -877,18 +872,41 @@ static __global__ void __launch_bounds__(4 * kInvTile * kInvTile)
       A[g][r][t] = x;
     }
     __syncthreads();
-    if (g == 3) {
-      const double uv = trail ? -A[1][r][t] : A[1][r][t];
-      x = fma(uv, A[2][c][t], x);
-    } else if (c > t && (g != 0 || r >= c)) {
+    if (c > t && (g != 0 || r >= c)) {
       x -= A[g][r][t] * A[0][c][t];
       if (g == 0 && c == t + 1 && r == c) pivot(c, x);
     }
     __syncthreads();
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && bad && info[col] == 0) info[col] = bad;
+  if (b == 0 && threadIdx.x == 0 && bad && info[col] == 0) info[col] = bad;
+  if (g == 1) panall[((int64_t)col * gridDim.x + b) * (Q * Q) + r * Q + c] = x;
+}
+
+// tile (bi, bj), bi >= bj, of the lower triangle: one thread per element
+static __global__ void __launch_bounds__(kInvTile * kInvTile)
+    k_inverse_update(int n, int nb, int k, int last, const double* __restrict__ srcall, double* __restrict__ dstall,
+                     const double* __restrict__ panall) {
+  constexpr int Q = kInvTile;
+  __shared__ double A[2][Q][Q + 1];
+  const int col = blockIdx.y;
+  const double* __restrict__ S = srcall + (int64_t)col * n * n;
+  double* __restrict__ O = dstall + (int64_t)col * n * n;
+  int bi = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+  while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
+  const int bj = (int)blockIdx.x - bi * (bi + 1) / 2;
+  const int r = threadIdx.x / Q, c = threadIdx.x % Q;
+  const bool trail = bi > k;  // the tile subtracts (else it adds)
+  const double* pan = panall + (int64_t)col * nb * (Q * Q) + threadIdx.x;
+  double x = (trail ? bj == k : bi == k) ? 0.0 : inverse_get(S, n, bi, bj, r, c);
+  const double u = pan[bi * (Q * Q)];
+  A[0][r][c] = trail ? -u : u;
+  A[1][r][c] = pan[bj * (Q * Q)];
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < Q; ++t) x = fma(A[0][r][t], A[1][c][t], x);
   const int i = bi * Q + r, j = bj * Q + c;
-  if (g == 3 && i < n && j < n) {
+  if (i < n && j < n) {
     O[(int64_t)i * n + j] = x;
     if (last && bi != bj) O[(int64_t)j * n + i] = x;
   }

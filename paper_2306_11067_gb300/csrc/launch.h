@@ -99,8 +99,9 @@ bool vtail_fits(int nlev);
 void launch_dense_setup(const LevelView<double>& L, int B, const double* lam2, double* M,
                         double* W, double* K, int* info, int max_blocks, cudaStream_t s);
 // K = M^{-1} of B symmetric positive definite n x n matrices (lower triangle
-// of M read; W is scratch of the same size, M keeps its values); info[b] = 0,
-// or the 1-based index of the first pivot that was not positive
+// of M read; W is scratch of B dense_inverse_scratch(n) values, M keeps its
+// values); info[b] = 0, or the 1-based index of the first pivot that was not positive
+int64_t dense_inverse_scratch(int64_t n);
 void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, int* info, cudaStream_t s);
 // the coarse operators of two fine ones on the same grid
 void launch_galerkin(const RapIn& in0, const RapIn& in1, int nvc, int nhc, double* out0, double* out1, cudaStream_t s);

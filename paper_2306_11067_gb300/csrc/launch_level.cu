@@ -457,14 +457,21 @@ void launch_dense_setup(const LevelView<double>& L, int B, const double* lam2, d
   launch_dense_inverse((int)nc, B, M, W, K, info, s);
 }
 
+int64_t dense_inverse_scratch(int64_t n) {
+  return n * n + (n + kInvTile - 1) / kInvTile * (kInvTile * kInvTile);
+}
+
 void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, int* info, cudaStream_t s) {
   LCMG_CUDA(cudaMemsetAsync(info, 0, sizeof(int) * B, s));
-  const int nb = (n + kInvTile - 1) / kInvTile;
+  const int nb = (n + kInvTile - 1) / kInvTile, threads = kInvTile * kInvTile;
+  double* pan = W + (int64_t)B * n * n;
   const double* src = M;
   for (int k = 0; k < nb; ++k) {  // the last step writes K
     double* dst = (nb - 1 - k) % 2 == 0 ? K : W;
-    klaunch(k_inverse_step, dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)B), dim3(4 * kInvTile * kInvTile), 0, s, n, k,
-            k == nb - 1 ? 1 : 0, src, dst, info);
+    klaunch(k_inverse_panel, dim3((unsigned)nb, (unsigned)B), dim3(2 * threads), 0, s, n, k, src, pan, info);
+    LCMG_LAUNCHED();
+    klaunch(k_inverse_update, dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)B), dim3(threads), 0, s, n, nb, k,
+            k == nb - 1 ? 1 : 0, src, dst, (const double*)pan);
     LCMG_LAUNCHED();
     src = dst;
   }
