@@ -374,7 +374,7 @@ static void build_hierarchy(lcmg_ctx& c) {
       in.g25 = f.gl.p;
       in2.g25 = f.ga.p;
     }
-    launch_galerkin(in, in2, g.nv, g.nh, gl, ga, c.stream);
+    launch_galerkin(in, in2, g.nv, g.nh, gl, ga, c.prm.precond == 1, c.maxblk, c.stream);
     // smoother copies: per-point rows of both parts (FP64 and FP32)
     const int gg = (int)std::min<int64_t>((kCoefStride * g.n + kBlock - 1) / kBlock, c.maxblk);
     klaunch(k_coef_pack<double>, dim3(gg), dim3(kBlock), 0, c.stream, g.n, gl, ga, g.cf64.need(kCoefStride * g.n));
@@ -2117,11 +2117,13 @@ int lcmg_set_params(lcmg_ctx* ctx, const lcmg_params* p) {
   lcmg::check_params(*p);
   const bool lev_change = p->levels != ctx->prm.levels || p->coarse_max != ctx->prm.coarse_max ||
                           p->coarsening != ctx->prm.coarsening;
+  // (the paper's method sums its Galerkin products in another order)
+  const bool hier_change = lev_change || (p->precond == 1) != (ctx->prm.precond == 1);
   const bool amg_change = lev_change || p->amg_coarse_max != ctx->prm.amg_coarse_max;
   ctx->prm = *p;
   ctx->maxblk = std::min(lcmg::kMaxBlocks, ctx->sms * 8);
   if (p->max_blocks > 0) ctx->maxblk = std::min(ctx->maxblk, p->max_blocks);
-  if (lev_change) ctx->hier_ok = false;
+  if (hier_change) ctx->hier_ok = false;
   if (amg_change) {
     ctx->am_ok = false;
     ctx->pm_levels = 0;

@@ -1046,6 +1046,50 @@ static __global__ void __launch_bounds__(kGalThreads)
   }
 }
 
+// The same product term by term, one thread per (coarse point, offset): for
+// the paper's own method (params.precond = 1), whose V(2,1) amplifies rounding
+// so strongly that at small lambda FGMRES stalls near 1e-9; another order of
+// these sums moved its solutions by 1e-8 there.
+static __global__ void __launch_bounds__(kBlock) k_galerkin_terms(RapIn in, int nvc, int nhc, double* __restrict__ out) {
+  const int64_t nc = (int64_t)nvc * nhc;
+  const int R = (in.part == 2) ? 2 : 1;
+  for (int64_t t = (int64_t)blockIdx.x * kBlock + threadIdx.x; t < nc * kStencil;
+       t += (int64_t)gridDim.x * kBlock) {
+    const int o = (int)(t / nc);
+    const int64_t P = t - (int64_t)o * nc;
+    const int J = (int)(P / nvc), I = (int)(P - (int64_t)J * nvc);
+    const int oi = o % 5 - 2, oj = o / 5 - 2;
+    const int It = I + oi, Jt = J + oj;
+    double sum = 0.0;
+    if (It >= 0 && It < nvc && Jt >= 0 && Jt < nhc) {
+      for (int b = 2 * J - 1; b <= 2 * J + 2; ++b) {
+        if (b < 0 || b >= in.nhf) continue;
+        const double wb = pw1(b, J, nhc);
+        for (int a = 2 * I - 1; a <= 2 * I + 2; ++a) {
+          if (a < 0 || a >= in.nvf) continue;
+          const double wab = wb * pw1(a, I, nvc);
+          const int64_t f = (int64_t)a + (int64_t)b * in.nvf;
+          for (int dj = -R; dj <= R; ++dj) {
+            const int d = b + dj;
+            if (d < 0 || d >= in.nhf) continue;
+            const double wd = pw1(d, Jt, nhc);
+            if (wd == 0.0) continue;
+            for (int di = -R; di <= R; ++di) {
+              const int c = a + di;
+              if (c < 0 || c >= in.nvf) continue;
+              if (in.part != 2 && di != 0 && dj != 0) continue;
+              const double wc = pw1(c, It, nvc);
+              if (wc == 0.0) continue;
+              sum += wab * in.coef(di, dj, f, a, b) * wc * wd;
+            }
+          }
+        }
+      }
+    }
+    out[t] = sum;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // PCG recurrences.  Per-column scalars live in device memory; a column
 // whose active flag is 0 is frozen (converged, stopped, or waiting for its

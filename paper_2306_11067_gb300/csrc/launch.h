@@ -103,8 +103,9 @@ void launch_dense_setup(const LevelView<double>& L, int B, const double* lam2, d
 // values); info[b] = 0, or the 1-based index of the first pivot that was not positive
 int64_t dense_inverse_scratch(int64_t n);
 void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, int* info, cudaStream_t s);
-// the coarse operators of two fine ones on the same grid
-void launch_galerkin(const RapIn& in0, const RapIn& in1, int nvc, int nhc, double* out0, double* out1, cudaStream_t s);
+// the coarse operators of two fine ones on the same grid (terms: summed term by term)
+void launch_galerkin(const RapIn& in0, const RapIn& in1, int nvc, int nhc, double* out0, double* out1, bool terms,
+                     int max_blocks, cudaStream_t s);
 
 template <class T, class TX>
 int launch_update_xr(int64_t n, int B, const ColState& st, const T* p, const T* q, TX* x, T* r,

@@ -477,7 +477,17 @@ void launch_dense_inverse(int n, int B, const double* M, double* W, double* K, i
   }
 }
 
-void launch_galerkin(const RapIn& in0, const RapIn& in1, int nvc, int nhc, double* out0, double* out1, cudaStream_t s) {
+void launch_galerkin(const RapIn& in0, const RapIn& in1, int nvc, int nhc, double* out0, double* out1, bool terms,
+                     int max_blocks, cudaStream_t s) {
+  if (terms) {
+    const int64_t work = (int64_t)nvc * nhc * kStencil;
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + kBlock - 1) / kBlock, max_blocks));
+    klaunch(k_galerkin_terms, dim3(g), dim3(kBlock), 0, s, in0, nvc, nhc, out0);
+    LCMG_LAUNCHED();
+    klaunch(k_galerkin_terms, dim3(g), dim3(kBlock), 0, s, in1, nvc, nhc, out1);
+    LCMG_LAUNCHED();
+    return;
+  }
   const unsigned tiles = (unsigned)((nvc + 31) / 32) * (unsigned)((nhc + kGalTJ - 1) / kGalTJ);
   klaunch(k_galerkin, dim3(tiles, 5, 2), dim3(kGalThreads), 0, s, in0, in1, nvc, nhc, out0, out1);
   LCMG_LAUNCHED();
