@@ -53,6 +53,26 @@ def test_cycle_in_strips_matches_its_model(n_v, n_h, levels, cols, smoother):
     s.close()
 
 
+@pytest.mark.parametrize("n_v,n_h,levels,cols", [(512, 384, 6, 1), (256, 176, 5, 2), (20, 12, 2, 1)])
+def test_fp64_cycle_in_tiles_of_every_size(n_v, n_h, levels, cols):
+    """k_vdown64 / k_vup64 with 8, 4 and 2 coarse points a side, against the oracle's
+    cycle to 1e-12 (FP64 rounding, summed in other orders)."""
+    s = Solver(n_v, n_h, levels=levels, nu=1)
+    s.set_forward_stencil(pg.gaussian_psf(2, 1.0))
+    d = pg.random_weights(ops.n_edges(n_v, n_h), 9, d_min=0.05)
+    s.set_weights(d)
+    R = pg.rng(4).standard_normal((cols, n_v * n_h))
+    rd = torch.tensor(R, device="cuda", dtype=torch.float64)
+    zd = torch.empty_like(rd)
+    diag = L.lcmg_get_diag(s.ctx, n_v * n_h)
+    H = mg.build_hierarchy(mg.weighted_laplacian(ops.gradient(n_v, n_h), d), sp.diags(diag), n_v, n_h, levels)
+    L.lcmg_apply_vcycle_dev(s.ctx, np.full(cols, 0.3), rd, zd)
+    for k in range(cols):
+        ref = mg.VCycle(H, 0.3, nu=1)(R[k])
+        assert np.linalg.norm(zd[k].cpu().numpy() - ref) <= 1e-12 * np.linalg.norm(ref)
+    s.close()
+
+
 @pytest.mark.parametrize("n_v,n_h,levels", [(140, 72, 3), (12, 10, 2), (4, 130, 2), (256, 6, 2)])
 def test_galerkin_tiles(n_v, n_h, levels):
     s = Solver(n_v, n_h, levels=levels)
