@@ -99,17 +99,17 @@ Band<T> make_band(const SepPass& p, const T* d_dev) {
 
 // blocks of a banded pass resident at once on the current device
 template <class K>
-static int band_resident(K kern, size_t smem) {
+static int band_resident(K kern, size_t smem, int threads = kBandThreads) {
   static std::mutex mu;
-  static std::map<std::pair<const void*, std::pair<int, size_t>>, int> cache;
+  static std::map<std::pair<std::pair<const void*, int>, std::pair<int, size_t>>, int> cache;
   int dev = 0;
   LCMG_CUDA(cudaGetDevice(&dev));
-  const auto key = std::make_pair(reinterpret_cast<const void*>(kern), std::make_pair(dev, smem));
+  const auto key = std::make_pair(std::make_pair(reinterpret_cast<const void*>(kern), threads), std::make_pair(dev, smem));
   std::lock_guard<std::mutex> lock(mu);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
   int nb = 0, sms = 0;
-  LCMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kBandThreads, smem));
+  LCMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem));
   LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (nb < 1) throw CudaError("banded pass does not fit on an SM");
   cache[key] = nb * sms;
@@ -198,11 +198,13 @@ template <class T, class TO, int DIR, int EPI>
 static int band_direct(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop,
                        const T* P, const T* C, const double* lam2, const double* bvec, double* part, int max_blocks,
                        cudaStream_t s) {
-  auto k = k_band_direct<T, TO, DIR, EPI>;
   const int64_t n = (int64_t)nv * nh;
-  // small images in blocks of two warps, so that they spread over more SMs
+  // small images in blocks of two warps, so that they spread over more SMs,
+  // with more taps in flight per warp
   const int threads = n <= 64 * 1024 ? 64 : kBandThreads;
-  const int blocks = clamp_blocks((n + threads - 1) / threads, std::min(max_blocks, band_resident(k, 0)));
+  constexpr int kSmallU = 16, kLargeU = sizeof(T) == 8 ? 8 : 16;
+  auto k = threads == 64 ? k_band_direct<T, TO, DIR, EPI, kSmallU> : k_band_direct<T, TO, DIR, EPI, kLargeU>;
+  const int blocks = clamp_blocks((n + threads - 1) / threads, std::min(max_blocks, band_resident(k, 0, threads)));
   klaunch(k, dim3((unsigned)blocks, (unsigned)B), dim3(threads), 0, s, nv, nh, B, bd, in, out, fop, P, C, lam2, bvec,
           part);
   LCMG_LAUNCHED();
