@@ -929,7 +929,7 @@ def main_deblur(args, world, rank, local):
     it_ms = sum(s_["iterate_ms"] for s_ in st)
     b_its = sum(s_["batch_iterations"] for s_ in st)
     band = {
-        "kernel": "k_band (separable A^T A: u = (I (x) T_v) p along i, then q = (T_h (x) I) u + lam^2 L^T W L p "
+        "kernel": "k_band_line + k_band_rows (separable A^T A: u = (I (x) T_v) p along i, then q = (T_h (x) I) u + lam^2 L^T W L p "
                   "with p.q along j; 61 taps each, FP32)",
         "bound": "hbm", "unit": "GB/s", "peak": peak, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
         "achieved": (op_bytes / (op_ms / 1e3) / 1e9) if op_ms > 0 else None,
