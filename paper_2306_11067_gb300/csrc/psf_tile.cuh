@@ -23,7 +23,10 @@
 namespace lcmg {
 
 constexpr int kPsfTI = 32;                 // points along i per tile
-constexpr size_t kPsfSmem = 48 * 1024;     // larger PSFs keep one output per thread
+constexpr int kPsfWarps = 8;               // most warps per block
+// Dynamic shared memory of a block without an opt-in: 48 KB less the kernel's
+// own array (the warps' partial sums).  Larger PSFs keep one output per thread.
+constexpr size_t kPsfSmem = 48 * 1024 - kPsfWarps * sizeof(double);
 
 // epilogues, as of the banded passes
 enum : int { PSF_STORE = 0, PSF_NORMAL = 1 };
@@ -35,13 +38,13 @@ inline size_t psf_smem(int rv, int rh, int tj) {
 }
 
 template <int TRANS, int EPI>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(32 * kPsfWarps)
     k_psf_tile(PsfArgs a, const float* __restrict__ psf, int B, const float* __restrict__ in, float* __restrict__ out,
                FineOp<float> fop, const float* __restrict__ P, const double* __restrict__ lam2,
                double* __restrict__ part) {
   using Quad = Pack<float>;
   extern __shared__ __align__(16) float psf_raw[];
-  __shared__ double sred[8];
+  __shared__ double sred[kPsfWarps];
   const int nv = a.nv, nh = a.nh, ku = 2 * a.rv + 1, kw = 2 * a.rh + 1, KU = psf_padded(ku), PW = kPsfTI + KU;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int tj = blockDim.x >> 3, li = threadIdx.x & 7, jl = threadIdx.x >> 3;
