@@ -779,38 +779,29 @@ __global__ void __launch_bounds__(kBlock)
 // itself rather than wait for a third launch) and k_inverse_update advances
 // every tile with two of the panels.
 //
-// What bounds it: the chain of pivots (square root and reciprocal, about 80
-// cycles per FP64 operation) at small n, so little else stands in it: the
-// pivot block and the panel have 256 threads each, a column's threads lie in
-// different SM quarters for the two solves, and a division is three
-// operations from the pivot's reciprocal; at large n the FP64 pipe (less than
-// two multiply-adds per clock and SM) of the updates.  A step reads `src` and
-// writes `dst` (the pivot row and column are read by every panel).
+// What bounds it: the chain of pivots (a square root, a quotient and a
+// multiply-add each, of dependent FP64 operations of some 80 cycles) at small
+// n, so little else stands in it: the pivot block and the panel have 256
+// threads each, and a column's threads lie in different SM quarters for the
+// two solves; at large n the FP64 pipe (less than two multiply-adds per clock
+// and SM) of the updates.  A step reads `src` and writes `dst` (the pivot row
+// and column are read by every panel).
 // info[col] = the 1-based index of the first pivot that was not positive.
 //
-// Measured on GB300, per step, against one launch whose every tile solved
-// both of its panels again: n = 256 18.7 -> 15.4 + 2.8 us, n = 567 61 -> 15.5 + 7.2 us.
-// (One block per column that did all of it in
-// global memory took 123 ms at n = 567; the values are the same bit for bit.)
+// The square root and the quotients are the correctly rounded ones of the
+// library, so the values are those of the unblocked steps bit for bit.
+// (Multiplying by one reciprocal per pivot took 27.8 us per step of 567
+// points where the quotients take 36.1, launches included, but its rounding
+// left a solution of the 256 x 256 CT system 1.1e-8 from the oracle's, where
+// the quotients stay below 1e-8.)
+//
+// Measured on GB300, panel + update of a step: n = 160 23.9 + 4.1 us, n = 256
+// 23.8 + 4.2, n = 567 24.1 + 8.5.  One launch whose every tile solved both of
+// its panels again took 18.7 us at 256 and 61 us at 567 with cheaper, not
+// always correctly rounded roots and quotients (the panel 16.9 us with
+// those); one block per column that did all of it in global memory 123 ms at
+// n = 567.
 constexpr int kInvTile = 16;
-
-// sqrt(a) and its reciprocal, both rounded to nearest: an FP32 seed, one
-// third-order step for 1 / sqrt(a), then one residual correction of each
-// (the divisions below need the correctly rounded reciprocal).  Outside the
-// FP32 range the library's operations.
-__device__ __forceinline__ void pivot_root(double a, double& root, double& recip) {
-  if (a > 1e-36 && a < 1e36) {
-    const double y0 = (double)rsqrtf((float)a);
-    const double e = fma(-a * y0, y0, 1.0);
-    const double y = fma(y0, e * fma(e, 0.375, 0.5), y0);
-    const double s = a * y;
-    root = fma(0.5 * y, fma(-s, s, a), s);
-    recip = fma(y, fma(-root, y, 1.0), y);
-  } else {
-    root = sqrt(a);
-    recip = 1.0 / root;
-  }
-}
 
 // element (rr, cc) of tile (u, v), u >= v; a last partial tile is padded with
 // the rows and columns of the identity
@@ -826,7 +817,7 @@ static __global__ void __launch_bounds__(2 * kInvTile * kInvTile)
   constexpr int Q = kInvTile;
   // the pivot block (then its factor, lower triangle) and the panel
   __shared__ double A[2][Q][Q + 1];
-  __shared__ double s_piv, s_rec;
+  __shared__ double s_piv;
   __shared__ int bad;
   const int col = blockIdx.y, b = blockIdx.x;
   const double* __restrict__ S = srcall + (int64_t)col * n * n;
@@ -850,10 +841,7 @@ static __global__ void __launch_bounds__(2 * kInvTile * kInvTile)
       if (!bad) bad = k * Q + t + 1;
       a = 1.0;
     }
-    double root, recip;
-    pivot_root(a, root, recip);
-    s_piv = root;
-    s_rec = recip;
+    s_piv = sqrt(a);
   };
   if (threadIdx.x == 0) {
     bad = 0;
@@ -862,13 +850,8 @@ static __global__ void __launch_bounds__(2 * kInvTile * kInvTile)
   __syncthreads();
   for (int t = 0; t < Q; ++t) {
     if (c == t) {  // column t, final
-      const double piv = s_piv, rec = s_rec;
-      if (g == 0 && r == t) {
-        x = piv;
-      } else {  // x / piv to nearest (Markstein 1990: quotient, exact remainder, correction)
-        const double q = x * rec;
-        x = fma(fma(-q, piv, x), rec, q);
-      }
+      const double piv = s_piv;
+      x = g == 0 && r == t ? piv : x / piv;
       A[g][r][t] = x;
     }
     __syncthreads();
