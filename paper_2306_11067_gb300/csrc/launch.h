@@ -64,6 +64,8 @@ int launch_vdown(const LevelView<T>& L, int B, const T* lam2, const T* dinv, con
 template <class T>
 int launch_vup(const LevelView<T>& L, int B, const T* lam2, const T* dinv, const T* r, const T* ec,
                const T* zpre, T* zout, double* part, int nu, cudaStream_t s);
+// multiprocessors of the first device used (all of a system are alike)
+int sm_count();
 // kr = lam2 gl + ga, the rows of K(lambda) of a coarse level of n points
 void launch_rows64(int64_t n, const double* gl, const double* ga, double lam2, double* kr, int max_blocks,
                    cudaStream_t s);

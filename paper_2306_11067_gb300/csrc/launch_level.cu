@@ -71,15 +71,14 @@ void launch_residual(const LevelView<T>& L, int B, const T* lam2, const T* r, co
   LCMG_LAUNCHED();
 }
 
-// multiprocessors of the first device used (all of a system are alike)
-static int sm_count() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
+int sm_count() {
+  static const int count = [] {
+    int dev = 0, sms = 0;
     LCMG_CUDA(cudaGetDevice(&dev));
     LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return sms;
+    return sms;
+  }();
+  return count;
 }
 
 // Grid of a tile kernel: every tile once, at most the blocks resident at

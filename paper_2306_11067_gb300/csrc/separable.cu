@@ -132,6 +132,23 @@ static int band_tiles(int nv, int nh, int B, const Band<T>& bd, const T* in, TO*
   return blocks;
 }
 
+// the tap counts of the A^T A passes of radii 4, 9 and 15 compiled in (the
+// passes of an iteration); the others run in chunks of 8 taps
+template <class T, int DIR, int EPI>
+constexpr bool kBandCompiled = EPI != BAND_RESID2 && !(std::is_same<T, double>::value && DIR == 1 && EPI == BAND_STORE);
+template <class T, class TO, int DIR, int EPI, class... A>
+static int band_tiles_any(int nv, int nh, int B, const Band<T>& bd, A... args) {
+  if constexpr (kBandCompiled<T, DIR, EPI>) {
+    switch (2 * bd.H + 1) {
+      case 17: return band_tiles<T, TO, DIR, EPI, 17>(nv, nh, B, bd, args...);
+      case 37: return band_tiles<T, TO, DIR, EPI, 37>(nv, nh, B, bd, args...);
+      case 61: return band_tiles<T, TO, DIR, EPI, 61>(nv, nh, B, bd, args...);
+      default: break;
+    }
+  }
+  return band_tiles<T, TO, DIR, EPI, 0>(nv, nh, B, bd, args...);
+}
+
 // k_band_line and k_band_rows: the tap count rounded up to a compiled one
 template <class F>
 static int by_taps(int taps, F&& f) {
@@ -170,17 +187,19 @@ static int band_rows(int nv, int nh, const Band<float>& bd, const float* in, flo
 
 // opt k_band and k_band_rows into their shared memory on the current device
 // (outside stream capture)
-template <int DIR, int EPI, int TAPS>
+template <class T, int DIR, int EPI, int TAPS>
 static void band_optin() {
-  const int bytes = (int)band_smem_bytes<float>((2 * kBandMaxH + 1 + kBandChunk - 1) / kBandChunk);
-  LCMG_CUDA(cudaFuncSetAttribute(k_band<float, float, DIR, EPI, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  const int bytes = (int)band_smem_bytes<T>((2 * kBandMaxH + 1 + kBandChunk - 1) / kBandChunk);
+  LCMG_CUDA(cudaFuncSetAttribute(k_band<T, T, DIR, EPI, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
 }
-template <int DIR, int EPI>
+template <class T, int DIR, int EPI>
 static void band_optin_taps() {
-  band_optin<DIR, EPI, 0>();
-  band_optin<DIR, EPI, 17>();
-  band_optin<DIR, EPI, 37>();
-  band_optin<DIR, EPI, 61>();
+  band_optin<T, DIR, EPI, 0>();
+  if constexpr (kBandCompiled<T, DIR, EPI>) {
+    band_optin<T, DIR, EPI, 17>();
+    band_optin<T, DIR, EPI, 37>();
+    band_optin<T, DIR, EPI, 61>();
+  }
 }
 void prepare_band() {
   for (int taps : {17, 25, 37, 49, 61, 65})
@@ -190,8 +209,13 @@ void prepare_band() {
                                      (int)sizeof(float) * rows_floats(TAPS)));
       return 0;
     });
-  band_optin_taps<0, BAND_STORE>();
-  band_optin_taps<1, BAND_NORMAL>();
+  band_optin_taps<float, 0, BAND_STORE>();
+  band_optin_taps<float, 1, BAND_NORMAL>();
+  band_optin_taps<double, 0, BAND_STORE>();
+  band_optin_taps<double, 1, BAND_STORE>();
+  band_optin_taps<double, 1, BAND_NORMAL>();
+  band_optin_taps<double, 1, BAND_RESID2>();
+  band_optin_taps<double, 1, BAND_TRUERES>();
 }
 
 template <class T, class TO, int DIR, int EPI>
@@ -220,6 +244,26 @@ static int band_direct(int nv, int nh, int B, const Band<T>& bd, const T* in, TO
 constexpr int64_t kBandDirectMax = 440 * 440;
 constexpr int64_t kBandDirectMaxTiles = 256 * 256;  // ... where the alternative is k_band
 
+// Many columns in FP64: interleaved columns put the samples of neighbouring
+// points 8 B bytes apart, and one output per thread fetches a 32-byte sector
+// for each of them at every tap, where the tiles of k_band (32 x 128 outputs)
+// fetch it once.  Along the contiguous axis that costs most where the distance
+// is a multiple of the 128-byte line; along the strided one more with every
+// column.  The tiles in turn leave part of the GPU idle where they are ragged
+// or don't make the same number for every SM: `used` is the share of their
+// outputs that count.  Measured on GB300 in an iteration, one output per
+// thread / tiles, along i and along j: 256 x 256, 37 taps, 16 columns 145 / 116
+// and 162 / 145 us, 32 columns 277 / 212 and 311 / 264, 24 columns 141 / 165
+// and 223 / 206; 512 x 512, 61 taps, 16 columns 857 / 567 and 924 / 652, 8
+// columns 255 / 319 and 308 / 364; 128 x 128, 37 taps, 16 columns 47 / 67 and
+// 49 / 84; 320 x 320, 61 taps, 16 columns (used 0.66) 340 / 330 and 366 / 371.
+static bool band64_in_tiles(int dir, int nv, int nh, int B) {
+  const int len = dir == 0 ? nv : nh, lines = dir == 0 ? nh : nv, sms = sm_count();
+  const int64_t tiles = (int64_t)((len + kBandSeg - 1) / kBandSeg) * ((lines + kBandLines - 1) / kBandLines) * B;
+  const double used = (double)nv * nh * B / ((double)((tiles + sms - 1) / sms * sms) * (kBandSeg * kBandLines));
+  return used >= 0.75 && (dir == 0 ? B % 16 == 0 : B * used >= 11.5);
+}
+
 template <class T, class TO, int DIR, int EPI>
 int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, const FineOp<T>& fop, const T* P,
                 const T* C, const double* lam2, const double* bvec, double* part, int max_blocks, cudaStream_t s) {
@@ -234,14 +278,10 @@ int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, 
           return band_rows(nv, nh, bd, in, out, fop, P, lam2, part, max_blocks, s);
       }
     } else if (work > kBandDirectMaxTiles) {
-      // the tap counts of the A^T A passes of radii 4, 9 and 15 compiled in
-      switch (2 * bd.H + 1) {
-        case 17: return band_tiles<T, TO, DIR, EPI, 17>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-        case 37: return band_tiles<T, TO, DIR, EPI, 37>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-        case 61: return band_tiles<T, TO, DIR, EPI, 61>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-        default: return band_tiles<T, TO, DIR, EPI, 0>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
-      }
+      return band_tiles_any<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
     }
+  } else if (band64_in_tiles(DIR, nv, nh, B)) {
+    return band_tiles_any<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
   }
   return band_direct<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
 }

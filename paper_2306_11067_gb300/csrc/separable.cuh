@@ -20,7 +20,8 @@
 // the contiguous axis (DIR 0) or the strided axis (DIR 1): k_band_direct (one
 // output per thread; FP64, and small FP32 images), k_band_line (DIR 0) and
 // k_band_rows (DIR 1) for one column of a large FP32 image, and k_band
-// (either axis) for large FP32 batches of several columns.  DIR 1 is the
+// (either axis) for large batches of several columns in FP32 and of many (14
+// or more) in FP64.  DIR 1 is the
 // second pass of the normal operator and fuses its epilogue: the lam^2 L^T W
 // L p term, the store and the per-block partial sums of p.q (or of the true
 // residual, or of ||A x - b||^2).
@@ -320,7 +321,8 @@ __global__ void __launch_bounds__(32 * kRowWarps)
   }
 }
 
-// ---- large FP32 batches of several columns, and lines that are not a multiple of 4
+// ---- large FP32 batches of several columns, lines that are not a multiple of 4,
+// ---- and wide FP64 batches
 // A block filters tiles of 32 lines x 128 outputs of one column, staged in shared
 // memory.  At 512 x 512, 4 columns, 37 taps it takes 9.6 + 13.5 us; forms of the
 // two kernels above that read single interleaved elements took 12.6 + 16.8.
