@@ -411,7 +411,10 @@ LevelView<float> view<float>(const lcmg_ctx& c, int k) {
   if (c.h16_on) {
     v.h16 = true;
     v.fh = FineOpH{l.nv, l.nh, c.h_ws.p, c.h_we.p, c.h_ga.p, (float)(1.0 / c.hw_scale), (float)(1.0 / c.hg_scale)};
-    v.ch = CoarseOpH{l.nv, l.nh, l.n, l.hrows.p, l.hc.p, (float)(1.0 / l.hscale)};
+    if (c.prm.nu == 1)
+      v.ch = CoarseOpH{l.nv, l.nh, l.n, l.hrows.p, l.hc.p, (float)(1.0 / l.hscale)};
+    else
+      v.cr = CoarseRowsH{l.nv, l.nh, l.n, l.hrows.p, l.hc.p, (float)(1.0 / l.hscale)};
   }
   return v;
 }
@@ -719,8 +722,9 @@ struct Batch {
         Level& g = c.lev[k];
         g.hscale = half_scale(l2[0] * g.glmax + g.gamax);
         const int gg = (int)std::min<int64_t>((g.n + kBlock - 1) / kBlock, c.maxblk);
-        klaunch(k_compact_rows, dim3(gg), dim3(kBlock), 0, s, g.nv, g.nh, g.n, (const double*)g.gl.p,
-                (const double*)g.ga.p, l2[0], g.hscale, (const float*)g.hs.p, g.hrows.p, g.hc.p);
+        klaunch(c.prm.nu == 1 ? k_compact_rows<false> : k_compact_rows<true>, dim3(gg), dim3(kBlock), 0, s, g.nv, g.nh,
+                g.n, (const double*)g.gl.p, (const double*)g.ga.p, l2[0], g.hscale, (const float*)g.hs.p, g.hrows.p,
+                g.hc.p);
         LCMG_LAUNCHED();
       }
       c.h16_on = true;

@@ -98,11 +98,18 @@ struct FineOpH {
 // Coarse level in FP16: the off-diagonal coefficients of K(lam) for the
 // offsets o = (di+2) + 5 (dj+2) in increasing o, o = 12 left out, scaled by
 // 2^e, and per point the diagonal in the same units (the row sum of G_A
-// minus the stored off-diagonals).  The coefficients of 64 points of a grid
-// row lie together, [row j][block of 64 along i][24][64], so a warp reads
-// one coefficient of 64 points as one 128-byte line, the 24 of them at
-// fixed distances from one address.
-struct CoarseOpH {
+// minus the stored off-diagonals).  Two layouts, one per form of the cycle:
+//
+//  * one sweep (row streaming, vcoarse.cuh): the coefficients of 64 points of
+//    a grid row lie together, [row j][block of 64 along i][24][64], so a warp
+//    reads one coefficient of 64 points as one 128-byte line, the 24 of them
+//    at fixed distances from one address;
+//  * two sweeps (the tiles of vfused.cuh, one point per thread): the 24 of a
+//    point lie together, three 16-byte words (kByPoint).  24 two-byte loads
+//    per point made a cycle with two sweeps 5 to 13% slower: 1024 x 1024 156
+//    -> 174 us, four columns of 512 x 512 164 -> 180 us on GB300.
+template <bool kByPoint>
+struct CoarseH16 {
   int nv, nh;
   int64_t n;
   const __half* __restrict__ rows;
@@ -111,19 +118,30 @@ struct CoarseOpH {
   static constexpr int kRadius = 2;
 
   __host__ __device__ static int64_t blocks(int nv) { return (nv + 63) / 64; }
-  // elements of `rows`
+  // elements of `rows` (that of the blocks is at least 24 n)
   __host__ __device__ static int64_t size(int nv, int nh) { return blocks(nv) * nh * (24 * 64); }
-  // the first coefficient of point (i, j); coefficient h follows at + 64 h
+  // blocks: the first coefficient of point (i, j); coefficient h follows at + 64 h
   __device__ __forceinline__ const __half* at(int i, int j) const {
     return rows + ((int64_t)j * blocks(nv) + (i >> 6)) * (24 * 64) + (i & 63);
   }
 
-  // k[o] of K(lam) for o < 25 (lam2 is already in the stored rows)
-  __device__ __forceinline__ void coefs(int64_t p, float, float (&k)[28]) const {
-    const int j = (int)(p / nv), i = (int)(p - (int64_t)j * nv);
-    const __half* q = at(i, j);
+  // k[o] of K(lam) of point p = (i, j) for o < 25 (lam2 is already in the stored rows)
+  __device__ __forceinline__ void coefs(int64_t p, int i, int j, float (&k)[28]) const {
+    if constexpr (kByPoint) {
+      const uint4* q = reinterpret_cast<const uint4*>(rows) + 3 * p;
+      const uint4 q0 = q[0], q1 = q[1], q2 = q[2];
+      const uint32_t w[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
 #pragma unroll
-    for (int h = 0; h < kCompactOff; ++h) k[h < 12 ? h : h + 1] = __half2float(q[64 * h]) * sc;
+      for (int h = 0; h < 12; ++h) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[h]));
+        k[h < 6 ? 2 * h : 2 * h + 1] = f.x * sc;
+        k[h < 6 ? 2 * h + 1 : 2 * h + 2] = f.y * sc;
+      }
+    } else {
+      const __half* q = at(i, j);
+#pragma unroll
+      for (int h = 0; h < kCompactOff; ++h) k[h < 12 ? h : h + 1] = __half2float(q[64 * h]) * sc;
+    }
     k[12] = c[p] * sc;
     k[25] = k[26] = k[27] = 0;
   }
@@ -151,9 +169,9 @@ struct CoarseOpH {
     return acc;
   }
   template <class F>
-  __device__ __forceinline__ float apply_off(int64_t p, int i, int j, float lam2, F v) const {
+  __device__ __forceinline__ float apply_off(int64_t p, int i, int j, float, F v) const {
     float k[28];
-    coefs(p, lam2, k);
+    coefs(p, i, j, k);
     return apply_k(k, i, j, v);
   }
   template <class F>
@@ -161,19 +179,21 @@ struct CoarseOpH {
     auto vo = [&](int di, int dj) { return v((int64_t)(i + di) + (int64_t)(j + dj) * nv); };
     return apply_off(p, i, j, lam2, vo);
   }
-  __device__ __forceinline__ double l1(int64_t p, int, int, double) const {
+  __device__ __forceinline__ double l1(int64_t p, int i, int j, double) const {
     float k[28];
-    coefs(p, 0.f, k);
+    coefs(p, i, j, k);
     double s1 = 0;
     for (int o = 0; o < kStencil; ++o) s1 += fabs((double)k[o]);
     return s1;
   }
-  __device__ __forceinline__ double center(int64_t p, int, int, double) const {
+  __device__ __forceinline__ double center(int64_t p, int i, int j, double) const {
     float k[28];
-    coefs(p, 0.f, k);
+    coefs(p, i, j, k);
     return (double)k[12];
   }
 };
+using CoarseOpH = CoarseH16<false>;
+using CoarseRowsH = CoarseH16<true>;
 
 // dst = fp16(src * scale), rounded to nearest from FP64
 static __global__ void k_half_scaled(int64_t n, const double* __restrict__ src, double scale,
@@ -209,22 +229,23 @@ static __global__ void k_maxabs(int64_t n, const double* __restrict__ v, int ste
 
 // The rows of K(lam) = lam2 G_L + G_A in FP16 (x scale, a power of two) and
 // their diagonals: s the row sums of G_A.  One thread per point, so that
-// every access runs along the points; it was one thread per coefficient with
-// the 24 of a point together (48 bytes apart in every read of G_L and G_A).
+// every read of G_L and G_A runs along the points.
+template <bool kByPoint>
 static __global__ void __launch_bounds__(kBlock)
     k_compact_rows(int nv, int nh, int64_t n, const double* __restrict__ gl, const double* __restrict__ ga, double lam2,
                    double scale, const float* __restrict__ s, __half* __restrict__ rows, float* __restrict__ c) {
   const float fscale = (float)scale;
   for (int64_t p = (int64_t)blockIdx.x * kBlock + threadIdx.x; p < n; p += (int64_t)gridDim.x * kBlock) {
     const int j = (int)(p / nv), i = (int)(p - (int64_t)j * nv);
-    __half* q = rows + ((int64_t)j * CoarseOpH::blocks(nv) + (i >> 6)) * (24 * 64) + (i & 63);
+    __half* q = kByPoint ? rows + kCompactOff * p
+                         : rows + ((int64_t)j * CoarseOpH::blocks(nv) + (i >> 6)) * (24 * 64) + (i & 63);
     float sum = 0.f;
 #pragma unroll 8
     for (int h = 0; h < kCompactOff; ++h) {
       const int o = h < 12 ? h : h + 1;
       const double k = lam2 * gl[(int64_t)o * n + p] + ga[(int64_t)o * n + p];
       const __half v = __double2half(k * scale);
-      q[64 * h] = v;
+      q[(kByPoint ? 1 : 64) * h] = v;
       sum += __half2float(v);
     }
     c[p] = s[p] * fscale - sum;

@@ -23,7 +23,8 @@ struct LevelView {
   // level's operators below replace ws/we/ga and cf in the V-cycle
   bool h16 = false;
   FineOpH fh{};
-  CoarseOpH ch{};
+  CoarseOpH ch{};    // one sweep
+  CoarseRowsH cr{};  // two sweeps (the rows of ch are null then, and the other way round)
   // FP64, a batch whose columns share one lambda: the 25 coefficients of
   // K(lambda) (coarse levels, [25][n]), or null
   const T* kr = nullptr;

@@ -24,7 +24,8 @@ void launch_dinv(const LevelView<T>& L, int B, const double* lam2, int smoother,
       if (L.fine)
         klaunch(k_dinv<FineOpH, float>, dim3(g), dim3(kBlock), 0, s, L.fh, L.n, B, lam2, smoother, omega, dinv);
       else
-        klaunch(k_dinv<CoarseOpH, float>, dim3(g), dim3(kBlock), 0, s, L.ch, L.n, B, lam2, smoother, omega, dinv);
+        L.ch.rows ? klaunch(k_dinv<CoarseOpH, float>, dim3(g), dim3(kBlock), 0, s, L.ch, L.n, B, lam2, smoother, omega, dinv)
+                  : klaunch(k_dinv<CoarseRowsH, float>, dim3(g), dim3(kBlock), 0, s, L.cr, L.n, B, lam2, smoother, omega, dinv);
       LCMG_LAUNCHED();
       return;
     }
@@ -240,7 +241,7 @@ int launch_vdown(const LevelView<T>& L, int B, const T* lam2, const T* dinv, con
                     : vdown_one<FineOpH, float, 2>(L.fh, B, lam2, dinv, r, zpre, rc, ntx, nt, s);
       else
         g = nu == 1 ? vdown_h(L.ch, B, dinv, r, rc, s)
-                    : vdown_one<CoarseOpH, float, 2>(L.ch, B, lam2, dinv, r, zpre, rc, ntx, nt, s);
+                    : vdown_one<CoarseRowsH, float, 2>(L.cr, B, lam2, dinv, r, zpre, rc, ntx, nt, s);
       LCMG_LAUNCHED();
       return g;
     }
@@ -278,7 +279,7 @@ int launch_vup(const LevelView<T>& L, int B, const T* lam2, const T* dinv, const
                     : vup_one<FineOpH, float, 2>(L.fh, B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
       else
         g = nu == 1 ? vup_h(L.ch, B, dinv, r, ec, zout, s)
-                    : vup_one<CoarseOpH, float, 2>(L.ch, B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
+                    : vup_one<CoarseRowsH, float, 2>(L.cr, B, lam2, dinv, r, ec, zpre, zout, part, ntx, nt, s);
       LCMG_LAUNCHED();
       return g;
     }
