@@ -67,8 +67,8 @@ RECORDS = {
     "k_band": (os.path.join(ROOT, "profiles", "k_band_deblur2048_traffic.txt"),
                ("separable.cuh", "separable.cu", "kernels.cuh", "common.cuh")),
     "vcycle": (os.path.join(ROOT, "profiles", "vcycle_deblur2048_traffic.txt"),
-               ("vfine.cuh", "vcoarse.cuh", "vfused.cuh", "compact.cuh", "kernels.cuh", "launch_level.cu",
-                "common.cuh")),
+               ("vfine.cuh", "vcoarse.cuh", "vtail.cuh", "vfused.cuh", "compact.cuh", "kernels.cuh",
+                "launch_level.cu", "common.cuh")),
 }
 
 
@@ -943,7 +943,8 @@ def main_deblur(args, world, rank, local):
     }
     band["frac"] = band["achieved"] / peak if band["achieved"] else None
     vcyc = {
-        "kernel": "V(1,1) cycle, 10 levels: k_vdown / k_vup per level (FP16 smoother data) + k_coarse_solve",
+        "kernel": "V(1,1) cycle, 10 levels (FP16 smoother data): k_vfine_down_s / k_vfine_up_s on the finest, k_vdown_h or "
+                  "k_vdown_h1 / k_vup_h on the next five, k_vtail_h for the rest and the coarsest solve",
         "bound": "hbm", "unit": "GB/s", "peak": peak, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
         "achieved": (v_bytes / (v_ms / 1e3) / 1e9) if v_ms > 0 else None,
         "algorithmic_bytes_per_cycle": (v_bytes / v_cnt) if v_cnt else None,

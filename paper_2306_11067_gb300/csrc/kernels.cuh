@@ -1102,16 +1102,17 @@ __global__ void __launch_bounds__(kBlock)
 }
 
 // ---- one column: the updates with their scalars ---------------------------
-// What bounds the two kernels: HBM at large n (x, r read and written, p, q
-// read; z read, p read and written), the latency of the partial sums and of
+// What bounds the two kernels: the vectors' bytes at large n (x, r read and
+// written, p, q read; z read, p read and written), the latency of the partial sums and of
 // the first loads at small n.  So the vectors move in 16-byte words, two
 // words of each per thread in flight, the first two issued before the
 // partial sums are taken; and the grid is at most two blocks of 512 threads
 // per SM, since every block repeats the FP64 sums (the FP64 pipe runs at a
 // small fraction of the FP32 one), which four warps share.  Measured on
 // GB300 at 2048^2 in FP32, against scalar loads in a grid of four blocks of
-// 256 threads per SM whose first warp summed alone: 33.7 -> 14.0 us (the 101
-// MB take 14.8 from HBM) and 21.8 -> 9.7 us (50 MB, 7.4).
+// 256 threads per SM whose first warp summed alone: 33.7 -> 14.0 us and
+// 21.8 -> 9.7 us (the reads, 67 and 34 MB, take 9.9 and 4.9 at the copy rate; the
+// writes stay in L2; the rest is the partial sums ahead of the first store).
 //
 // At small n an FP64 warp instruction holds an SM for 19 cycles, so there are
 // few of them: blocks of 256 threads, the block's r.r combined through shared

@@ -85,7 +85,7 @@ int sm_count() {
 // Grid of a tile kernel: every tile once, at most the blocks resident at
 // once on the device and at most kMaxTileBlocks (rows of the partial sums).
 template <class K>
-static int tile_grid(K kern, int threads, int ntiles, size_t smem = 0) {
+static int tile_grid(K kern, int threads, int ntiles) {
   static std::mutex mu;
   static std::map<std::pair<const void*, int>, int> cache;
   int dev = 0;
@@ -96,10 +96,9 @@ static int tile_grid(K kern, int threads, int ntiles, size_t smem = 0) {
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(key);
     if (it == cache.end()) {
-      int nb = 0, sms = 0;
-      LCMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem));
-      LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-      it = cache.emplace(key, std::max(1, nb) * sms).first;
+      int nb = 0;
+      LCMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, 0));
+      it = cache.emplace(key, std::max(1, nb) * sm_count()).first;
     }
     wave = it->second;
   }
@@ -136,12 +135,7 @@ static int vup_one(const Op& op, int B, const T* lam2, const T* dinv, const T* r
 // 5.9 us; 1024 x 1024, mean of five 26.6 + 21.2 -> 14 + 10 us.
 template <class F>
 static int tiles64(int nvc, int nhc, int B, F&& f) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    LCMG_CUDA(cudaGetDevice(&dev));
-    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
+  const int sms = sm_count();
   auto nt = [](int n, int tc) { return (n + tc - 1) / tc; };
   int best = 8;
   int64_t least = INT64_MAX;
@@ -195,13 +189,7 @@ void launch_rows64(int64_t n, const double* gl, const double* ga, double lam2, d
 // reads two residual rows more than it produces).  Measured on GB300 at
 // 1024^2 points with 8, 16 and 24 warps: down 23.7, 18.4, 22.1 us.
 static int coarse_strip(int nsi, int nhc, int B) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    LCMG_CUDA(cudaGetDevice(&dev));
-    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  const int64_t per_col = std::max<int64_t>(1, ((int64_t)sms * kVcWarps) / ((int64_t)nsi * B));
+  const int64_t per_col = std::max<int64_t>(1, ((int64_t)sm_count() * kVcWarps) / ((int64_t)nsi * B));
   return std::max(1, std::min(16, (int)((nhc + per_col - 1) / per_col)));
 }
 template <class K, class... A>
@@ -354,12 +342,7 @@ void launch_vtail(const TailLevelIn* levels, int nlev, const double* kinv, int n
 // dot products it needs in FP64); blocks of 256 threads while they fit on as
 // many SMs, so that a short vector's FP64 work is spread
 static dim3 fused_update_grid(int64_t words, int max_blocks, int* threads) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    LCMG_CUDA(cudaGetDevice(&dev));
-    LCMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
+  const int sms = sm_count();
   *threads = words <= (int64_t)sms * (kUpdThreads / 2) ? kUpdThreads / 2 : kUpdThreads;
   const int64_t want = (words + *threads - 1) / *threads;
   return dim3((unsigned)std::max<int64_t>(1, std::min(want, (int64_t)std::min(2 * sms, max_blocks))));

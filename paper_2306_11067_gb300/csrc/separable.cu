@@ -286,15 +286,15 @@ int launch_band(int nv, int nh, int B, const Band<T>& bd, const T* in, TO* out, 
   return band_direct<T, TO, DIR, EPI>(nv, nh, B, bd, in, out, fop, P, C, lam2, bvec, part, max_blocks, s);
 }
 
-// Tiles of 8 rows in blocks of 64 threads while that leaves SMs idle, else of
-// 32 rows (the halo of 2 rh rows is staged per tile); one output per thread
+// Tiles of 8 rows in blocks of 64 threads while tiles of 32 would give an SM
+// less than two, else of 32 rows (the halo of 2 rh rows is staged per tile); one output per thread
 // where the PSF's tile does not fit in kPsfSmem (radii above 24 or so).
 template <int TRANS, int EPI>
 int launch_psf(const PsfArgs& a, const float* psf, int B, const float* in, float* out, const FineOp<float>& fop,
                const float* P, const double* lam2, double* part, int max_blocks, cudaStream_t s) {
   const int nti = (a.nv + kPsfTI - 1) / kPsfTI;
   auto tiles = [&](int tj) { return (int64_t)nti * ((a.nh + tj - 1) / tj); };
-  const int tj = tiles(32) * B < 304 || psf_smem(a.rv, a.rh, 32) > kPsfSmem ? 8 : 32;
+  const int tj = tiles(32) * B < 2 * sm_count() || psf_smem(a.rv, a.rh, 32) > kPsfSmem ? 8 : 32;
   const size_t smem = psf_smem(a.rv, a.rh, tj);
   if (smem <= kPsfSmem) {
     const int blocks = clamp_blocks(tiles(tj), max_blocks);

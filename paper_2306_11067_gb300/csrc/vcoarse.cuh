@@ -16,8 +16,10 @@
 // coarse columns (down) or 60 columns of z (up).  A row's 24 coefficients are
 // 24 loads of 128 bytes per warp at fixed distances, issued one row ahead.
 //
-// What bounds them: at 1024^2 points HBM (48 of the 61 or so bytes per point
-// are coefficients); below 256^2 the latency of a row's loads, so strips are
+// What bounds them: the latency of a row's loads (128 and 149 registers: 15
+// and 12 warps per SM; the largest stalls at every size), at 1024^2 points with
+// DRAM at half of its peak (48 of the 61 or so bytes per point are
+// coefficients); so on the smaller levels strips are
 // as short as it takes to give every SM 16 warps (a strip reads two rows more
 // than it produces).  The 16 x 16 tiles staged in shared memory that they
 // replace took about 860 warp instructions per 32 points (a 25-point stencil

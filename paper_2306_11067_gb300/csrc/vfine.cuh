@@ -212,9 +212,13 @@ __global__ void __launch_bounds__(kFineThreads)
 // The weights are zero on the last row and column and outside the grid, so
 // no step tests for the edge.
 //
-// What bounds them: HBM at 2048^2 points (46 and 63 MB per launch), below
-// 512^2 the latency of a row's loads; with one point per lane it was the
-// instructions (165 per warp and row of 30 points).  Measured on GB300 against
+// What bounds them: the latency of a row's loads, of which a lane has one row
+// (10 bytes a point, and e_c) ahead of its use, in 22 (down, 80 registers) or 15
+// (up, 126) warps per SM.  At 2048^2 points the largest stalls are those loads'
+// (4.9 and 2.5 warps per issue), 55% of the issue slots are taken and DRAM runs
+// at 26 and 22% of its peak: 42 and 46 MB, 6.2 and 6.8 us at the copy rate.
+// With one point per lane it was the instructions (165 per warp and row of
+// 30 points).  Measured on GB300 against
 // that form, down / up: 2048^2 27.4 / 34.9 -> 18.5 / 24.1 us, 512^2 in four
 // columns 12.6 / 13.4 -> 8.0 / 10.4 us, 256^2 3.9 / 3.9 -> 3.5 / 3.8 us.  With as
 // many strips as 16 / 8, 24 / 16 and 32 / 32 warps per SM: 23.2 / 25.4, 18.3 /

@@ -16,7 +16,7 @@
 // A level of 32 x 32 points is 4 tiles of 8 x 8 coarse points, so 4 SMs
 // worked on it; smaller tiles compute more halo points in all but spread
 // them over the SMs, and the launcher takes the tile side with the fewest
-// residual points on the busiest SM (vt64_side).  The sums per point are
+// residual points on the busiest SM (tiles64).  The sums per point are
 // those of vfused.cuh in the same order.
 #pragma once
 #include <type_traits>
