@@ -779,28 +779,26 @@ __global__ void __launch_bounds__(kBlock)
 // itself rather than wait for a third launch) and k_inverse_update advances
 // every tile with two of the panels.
 //
-// What bounds it: the chain of pivots (a square root, a quotient and a
-// multiply-add each, of dependent FP64 operations of some 80 cycles) at small
-// n, so little else stands in it: the pivot block and the panel have 256
-// threads each, and a column's threads lie in different SM quarters for the
-// two solves; at large n the FP64 pipe (less than two multiply-adds per clock
-// and SM) of the updates.  A step reads `src` and writes `dst` (the pivot row
-// and column are read by every panel).
+// What bounds it: the chain of pivots at small n (a square root of 590 cycles,
+// a quotient of 575 and a multiply-add of 65 each), so little else stands in
+// it: the pivot block and the panel have 256 threads each, and a column's
+// threads lie in different SM quarters for the two solves; at large n the FP64
+// pipe (less than two multiply-adds per clock and SM) of the updates.  A step
+// reads `src` and writes `dst` (the pivot row and column are read by every
+// panel).
 // info[col] = the 1-based index of the first pivot that was not positive.
 //
 // The square root and the quotients are the correctly rounded ones of the
 // library, so the values are those of the unblocked steps bit for bit.
-// (Multiplying by one reciprocal per pivot took 27.8 us per step of 567
-// points where the quotients take 36.1, launches included, but its rounding
-// left a solution of the 256 x 256 CT system 1.1e-8 from the oracle's, where
-// the quotients stay below 1e-8.)
+// (One reciprocal per pivot and products round twice: a solution of the 256 x
+// 256 CT system came out 1.1e-8 from the oracle's, where the quotients stay
+// below 1e-8.)
 //
-// Measured on GB300, panel + update of a step: n = 160 23.9 + 4.1 us, n = 256
-// 23.8 + 4.2, n = 567 24.1 + 8.5.  One launch whose every tile solved both of
-// its panels again took 18.7 us at 256 and 61 us at 567 with cheaper, not
-// always correctly rounded roots and quotients (the panel 16.9 us with
-// those); one block per column that did all of it in global memory 123 ms at
-// n = 567.
+// Measured on GB300, panel + update of a step: n = 160 17.1 + 4.1 us, n = 256
+// 17.2 + 4.2, n = 567 17.2 + 8.4 (the panel 23.9 when zeros were divided too).
+// One launch whose every tile solved both of its panels again took 18.7 us at
+// 256 and 61 us at 567; one block per column that did all of it in global
+// memory 123 ms at n = 567.
 constexpr int kInvTile = 16;
 
 // element (rr, cc) of tile (u, v), u >= v; a last partial tile is padded with
@@ -850,8 +848,15 @@ static __global__ void __launch_bounds__(2 * kInvTile * kInvTile)
   __syncthreads();
   for (int t = 0; t < Q; ++t) {
     if (c == t) {  // column t, final
+      // zeros (and the pivot block's unused upper half) are kept out of the
+      // division, whose path for them takes 1670 cycles instead of 730; the
+      // empty asm keeps the compiler from folding the two selections away
       const double piv = s_piv;
-      x = g == 0 && r == t ? piv : x / piv;
+      const bool skip = x == 0.0 || (g == 0 && r <= t);
+      double num = skip ? 1.0 : x;
+      asm volatile("" : "+d"(num));
+      const double quot = num / piv;
+      x = g == 0 && r == t ? piv : skip ? x : quot;
       A[g][r][t] = x;
     }
     __syncthreads();
